@@ -292,6 +292,7 @@ struct F64Backend : Backend {
         a.dx = dx; a.dy = dy; a.half_dx = 0.5 * dx; a.half_dy = 0.5 * dy;
         a.inv_dx = 1.0 / dx; a.inv_dy = 1.0 / dy; a.dx_over_dy = dx / dy; a.dy_over_dx = dy / dx;
         a.beta = c->beta; a.inv_beta = 1.0 / c->beta; a.gx = c->grid.gx; a.gy = c->grid.gy;
+        a.fbeta = make_fixed_beta(c->beta);
         a.cfl_area = c->opt.cfl_tau * dx * dy;
         for (int b = 0; b < 3; ++b)
             for (int f = 0; f < 4; ++f) a.buf[b][f] = buf[b][f];

@@ -18,6 +18,7 @@
 #pragma once
 
 #include "ac_device.cuh"
+#include "ac_fixed_flux.cuh"
 
 namespace acgb {
 
@@ -71,6 +72,7 @@ struct SweepArgs {
     T alpha;                       // alpha_s of this stage
     T dx, dy, half_dx, half_dy, inv_dx, inv_dy, dx_over_dy, dy_over_dx;
     T beta, inv_beta, gx, gy;
+    FixedBeta fbeta;               // beta for the fixed-point Osher flux
     T cfl_area;                    // CFL_tau * |Omega|
     T *buf[3][4];                  // three state buffers: rho, rho u, rho v, p
     T *lev[4];                     // real-time level Q^n (rho, rho u, rho v, p)
@@ -397,7 +399,10 @@ stage_kernel(const SweepArgs<T> a) {
         // one flux call for both kinds: no divergence where a warp holds both
         // (2F: the divergence below takes the 1/2)
         T F[4];
-        riemann_flux<RS, T, true>(rL, nL, tL, pL, rR, nR, tR, pR, a.beta, a.inv_beta, F);
+        if (RS == kOsher && fixed_flux_ok(rL, nL, tL, pL, rR, nR, tR, pR))
+            osher_flux_fixed(rL, nL, tL, pL, rR, nR, tR, pR, a.fbeta, F);
+        else
+            riemann_flux<RS, T, true>(rL, nL, tL, pL, rR, nR, tR, pR, a.beta, a.inv_beta, F);
         T *fd = isx ? &sm.fx[0][fo] : &sm.fy[0][fo];
         const int fs = isx ? S::NXF : S::NYF;
         fd[0] = F[0];
