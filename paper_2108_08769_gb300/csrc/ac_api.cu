@@ -177,7 +177,7 @@ cudaError_t allow_f64_smem() {
 
 template <int TX, int TY, int RS = kOsher>
 cudaError_t launch_f64(const SweepArgs<double> &a, dim3 g, bool pdl, cudaStream_t s) {
-    return launch_pdl(pdl, stage_kernel<double, TX, TY, RS>, g, dim3(TX * TY), sizeof(StageSmem<double, TX, TY>), s,
+    return launch_pdl(pdl, stage_kernel<double, TX, TY, RS>, g, dim3(f64_threads(TX, TY)), sizeof(StageSmem<double, TX, TY>), s,
                       a);
 }
 
@@ -194,7 +194,7 @@ struct F64Backend : Backend {
         const F64Variant &m = kF64Variants[variant < 0 ? 0 : variant];
         tx = m.tx;
         ty = m.ty;
-        nt = m.tx * m.ty;
+        nt = f64_threads(m.tx, m.ty);
         return variant;
     }
 
@@ -292,8 +292,8 @@ struct F64Backend : Backend {
         a.dx = dx; a.dy = dy; a.half_dx = 0.5 * dx; a.half_dy = 0.5 * dy;
         a.inv_dx = 1.0 / dx; a.inv_dy = 1.0 / dy; a.dx_over_dy = dx / dy; a.dy_over_dx = dy / dx;
         a.beta = c->beta; a.inv_beta = 1.0 / c->beta; a.gx = c->grid.gx; a.gy = c->grid.gy;
-        a.fbeta = make_fixed_beta(c->beta);
         a.cfl_area = c->opt.cfl_tau * dx * dy;
+        set_flux_scales(a, c->beta, dx, dy);
         for (int b = 0; b < 3; ++b)
             for (int f = 0; f < 4; ++f) a.buf[b][f] = buf[b][f];
         for (int f = 0; f < 4; ++f) a.lev[f] = lev[f];

@@ -18,7 +18,6 @@
 #pragma once
 
 #include "ac_device.cuh"
-#include "ac_fixed_flux.cuh"
 
 namespace acgb {
 
@@ -72,7 +71,11 @@ struct SweepArgs {
     T alpha;                       // alpha_s of this stage
     T dx, dy, half_dx, half_dy, inv_dx, inv_dy, dx_over_dy, dy_over_dx;
     T beta, inv_beta, gx, gy;
+    int fixed;                     // the Osher flux may run in fixed point (beta and the cell sizes allow it)
     FixedBeta fbeta;               // beta for the fixed-point Osher flux
+    T hidx, hidy, phidx, phidy;    // 1/(2 dx), 1/(2 dy), and beta times them
+    FixedScale fhx, fhy, fphx, fphy;   // the same for the fixed-point flux
+    T inv_alpha, inv_cfl_area;
     T cfl_area;                    // CFL_tau * |Omega|
     T *buf[3][4];                  // three state buffers: rho, rho u, rho v, p
     T *lev[4];                     // real-time level Q^n (rho, rho u, rho v, p)
@@ -89,14 +92,35 @@ struct SweepArgs {
     int reuse;
 };
 
-// Frozen real-time term (Eq. bdf) of field f at index s, Q^{m} value qm:
-// (B0 Q^{m} + B1 Q^n + B2 Q^{n-1} + B3 Q^{n-2}) / dt, always in this order.
+// The constants of the fixed-point flux and of the scaled fluxes; alpha and cfl_area are set.
+inline void set_flux_scales(SweepArgs<double> &a, double beta, double dx, double dy) {
+    a.fixed = fixed_beta_ok(beta) && fixed_beta_ok(dx) && fixed_beta_ok(dy);
+    a.fbeta = make_fixed_beta(beta);
+    a.hidx = 0.5 / dx;
+    a.hidy = 0.5 / dy;
+    a.phidx = beta * a.hidx;
+    a.phidy = beta * a.hidy;
+    a.fhx = make_fixed_scale(a.hidx);
+    a.fhy = make_fixed_scale(a.hidy);
+    a.fphx = make_fixed_scale(a.phidx);
+    a.fphy = make_fixed_scale(a.phidy);
+    a.inv_alpha = double(a.s_max - a.stage + 1);
+    a.inv_cfl_area = 1.0 / a.cfl_area;
+}
+
+// Frozen real-time term (Eq. bdf) of field f at index s, Q^{m} value qm, Q^n
+// value ql: (B0 Q^{m} + B1 Q^n + B2 Q^{n-1} + B3 Q^{n-2}) / dt, always in this order.
 template <typename T>
-__device__ __forceinline__ T realtime_term(const SweepArgs<T> &a, T qm, int f, size_t s, T inv_dt) {
-    T r = fma(a.B[1], a.lev[f][s], a.B[0] * qm);
+__device__ __forceinline__ T realtime_term(const SweepArgs<T> &a, T qm, T ql, int f, size_t s, T inv_dt) {
+    if (a.order == 1) return (qm - ql) * inv_dt;   // Backward-Euler: B0 = 1, B1 = -1
+    T r = fma(a.B[1], ql, a.B[0] * qm);
     if (a.order >= 2) r = fma(a.B[2], a.lev1[f][s], r);
     if (a.order >= 3) r = fma(a.B[3], a.lev2[f][s], r);
     return r * inv_dt;
+}
+template <typename T>
+__device__ __forceinline__ T realtime_term(const SweepArgs<T> &a, T qm, int f, size_t s, T inv_dt) {
+    return realtime_term(a, qm, a.lev[f][s], f, s, inv_dt);
 }
 
 // Buffer roles within a pseudo-iteration: stage s reads `in` and writes
@@ -201,6 +225,11 @@ __device__ __forceinline__ T wall_ghost_sign(int gi, int gj, int nx, int ny, con
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Threads of the FP64 sweep's CTA on a TX x TY tile: one per cell, but 16 warps
+// on the 32x14 tile, whose two groups then have two warps on each of the four
+// SM sub-partitions (14 warps leave one warp alone on some).
+__host__ __device__ constexpr int f64_threads(int tx, int ty) { return tx == 32 && ty == 14 ? 512 : tx * ty; }
+
 template <typename T, int TX, int TY>
 struct StageSmem {
     static constexpr int RW = TX + 4, RH = TY + 4;   // tile + 2-cell halo
@@ -214,22 +243,36 @@ struct StageSmem {
     T gy[4][GW * GH];     // whole slopes along y
     T fx[4][NXF];         // x-face fluxes: mass, x-mom, y-mom, p/beta
     T fy[4][NYF];         // y-face fluxes
-    double red[4][TX * TY / 32];
+    double red[4][f64_threads(TX, TY) / 32];
 };
 
-// Tiles of 448 cells are sized to run one per SM: they may take the whole
-// register file (ptxas otherwise budgets for two CTAs per SM and recomputes
-// products to stay inside it).  Other shapes keep the compiler's choice.
-constexpr int f64_min_blocks(int nt) { return nt >= 448 ? 1 : 0; }
+// CTAs per SM the register allocation is asked to allow.  Tiles of 448 cells
+// run one per SM and take the whole register file; 256-thread tiles run three
+// (80 registers and a few spills: 558 us per pseudo-iteration of a 1024x512
+// tank, 660-706 us at two or four), so that the FP64-bound phases of one CTA
+// run beside the integer-bound faces of another; 128-thread tiles four.
+constexpr int f64_min_blocks(int nt) { return nt >= 448 ? 1 : nt == 256 ? 3 : nt == 128 ? 4 : 0; }
+
+// Named barriers of a CTA: wait for, or only signal, barrier id of n threads.
+__device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ void bar_arrive(int id, int n) {
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
 
 template <typename T, int TX, int TY, int RS = kOsher>
-__global__ void __launch_bounds__(TX * TY, f64_min_blocks(TX * TY))
+__global__ void __launch_bounds__(f64_threads(TX, TY), f64_min_blocks(TX * TY))
 stage_kernel(const SweepArgs<T> a) {
     using S = StageSmem<T, TX, TY>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     S &sm = *reinterpret_cast<S *>(smem_raw);
-    constexpr int NT = TX * TY;
+    constexpr int NT = f64_threads(TX, TY);
     constexpr int RW = S::RW, RH = S::RH, GW = S::GW, GH = S::GH;
+    // A 32x14 tile runs alone on its SM, so nothing else fills the FP64 unit
+    // while its faces keep the integer pipes busy.  Its warps therefore work in
+    // two groups, one per half of the rows, the second a phase behind: the
+    // first group's faces run beside the second's slopes, and its update
+    // beside the second's faces (256x256 tank: 105 -> 91 us per pseudo-iteration).
+    constexpr int GR = (TX == 32 && TY == 14) ? 2 : 1, NTG = NT / GR;
 
     pdl_trigger();
     pdl_wait();
@@ -247,46 +290,92 @@ stage_kernel(const SweepArgs<T> a) {
     const int tid = threadIdx.x;
     const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
 
+    // A tile whose halo lies inside the domain needs no ghost folding.  The
+    // ring's real-time inputs are loaded first and used last, and interior
+    // tiles load all their halo cells before the first is used, so that one
+    // round trip to memory covers them.
+    const bool interior = x0 >= 2 && x0 + TX + 2 <= nx && y0 >= 2 && y0 + TY + 2 <= ny;
+    const bool need_rt = (a.gradp == kGradNew) && a.realtime;
+    const bool reuse_now = a.reuse && a.stage > 1;   // fixed per-cell values from stage 1
+    constexpr int NR = (GW * GH + NT - 1) / NT, NW = (RW * RH + NT - 1) / NT;
+    T rt_q[NR][2], rt_l[NR][2];   // real-time terms (later stages) or Q^{m} and Q^n (stage 1) of rho u, rho v
+    int rt_s[NR], rt_f[NR];       // source cell and signs of the ring cell
+    if (need_rt) {
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            const int k = tid + r * NT;
+            rt_f[r] = 0;
+            if (k >= GW * GH) continue;
+            const int gi = x0 + (k % GW) - 1, gj = y0 + (k / GW) - 1;
+            if (interior) {
+                rt_s[r] = gj * nx + gi;
+            } else {
+                int nfx, tfx, nfy, tfy;
+                const int si = fold_axis(gi, nx, a.bc[0], a.bc[1], nfx, tfx);
+                const int sj = fold_axis(gj, ny, a.bc[2], a.bc[3], nfy, tfy);
+                rt_s[r] = sj * nx + si;
+                rt_f[r] = ((nfx + tfy) & 1) | (((nfy + tfx) & 1) << 1);
+            }
+            if (reuse_now) {
+                rt_q[r][0] = a.aux[2][rt_s[r]];
+                rt_q[r][1] = a.aux[3][rt_s[r]];
+            } else {
+                rt_q[r][0] = q0[1][rt_s[r]];
+                rt_q[r][1] = q0[2][rt_s[r]];
+                rt_l[r][0] = a.lev[1][rt_s[r]];
+                rt_l[r][1] = a.lev[2][rt_s[r]];
+            }
+        }
+    }
     // ---- 1. stage Q^{s-1} (+ two-cell halo, ghosts synthesised) as W ----
-    for (int k = tid; k < RW * RH; k += NT) {
-        const int gi = x0 + (k % RW) - 2, gj = y0 + (k / RW) - 2;
-        int nfx, tfx, nfy, tfy;
-        const int si = fold_axis(gi, nx, a.bc[0], a.bc[1], nfx, tfx);
-        const int sj = fold_axis(gj, ny, a.bc[2], a.bc[3], nfy, tfy);
-        const size_t s = (size_t)sj * nx + si;
-        const T r = qin[0][s];
-        T m = qin[1][s], n = qin[2][s];
-        if ((nfx + tfy) & 1) m = -m;
-        if ((nfy + tfx) & 1) n = -n;
+    auto put_w = [&](int k, T r, T m, T n, T p) {
         const T ir = Ar<T>::rcp(r);
         sm.w[0][k] = r;
         sm.w[1][k] = m * ir;
         sm.w[2][k] = n * ir;
-        sm.w[3][k] = qin[3][s];
+        sm.w[3][k] = p;
         sm.wir[k] = ir;
-    }
-    // ---- frozen real-time term of the momenta on the ring (Eq. bdf, BE) ----
-    const bool need_rt = (a.gradp == kGradNew) && a.realtime;
-    const bool reuse_now = a.reuse && a.stage > 1;   // fixed per-cell values from stage 1
-    if (need_rt) {
-        for (int k = tid; k < GW * GH; k += NT) {
-            const int gi = x0 + (k % GW) - 1, gj = y0 + (k / GW) - 1;
+    };
+    if (interior) {
+        T in4[NW][4];
+        const int base = (y0 - 2) * nx + (x0 - 2);
+#pragma unroll
+        for (int r = 0; r < NW; ++r) {
+            const int k = tid + r * NT;
+            if (k >= RW * RH) continue;
+            const int s = base + (k / RW) * nx + k % RW;
+#pragma unroll
+            for (int f = 0; f < 4; ++f) in4[r][f] = qin[f][s];
+        }
+#pragma unroll
+        for (int r = 0; r < NW; ++r)
+            if (tid + r * NT < RW * RH) put_w(tid + r * NT, in4[r][0], in4[r][1], in4[r][2], in4[r][3]);
+    } else {
+        for (int k = tid; k < RW * RH; k += NT) {
+            const int gi = x0 + (k % RW) - 2, gj = y0 + (k / RW) - 2;
             int nfx, tfx, nfy, tfy;
             const int si = fold_axis(gi, nx, a.bc[0], a.bc[1], nfx, tfx);
             const int sj = fold_axis(gj, ny, a.bc[2], a.bc[3], nfy, tfy);
             const size_t s = (size_t)sj * nx + si;
-            T rx, ry;
-            if (reuse_now) {
-                rx = a.aux[2][s];
-                ry = a.aux[3][s];
-            } else {
-                rx = realtime_term(a, q0[1][s], 1, s, inv_dt);
-                ry = realtime_term(a, q0[2][s], 2, s, inv_dt);
+            T m = qin[1][s], n = qin[2][s];
+            if ((nfx + tfy) & 1) m = -m;
+            if ((nfy + tfx) & 1) n = -n;
+            put_w(k, qin[0][s], m, n, qin[3][s]);
+        }
+    }
+    // ---- frozen real-time term of the momenta on the ring (Eq. bdf) ----
+    if (need_rt) {
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            const int k = tid + r * NT;
+            if (k >= GW * GH) continue;
+            T rx = rt_q[r][0], ry = rt_q[r][1];
+            if (!reuse_now) {
+                rx = realtime_term(a, rx, rt_l[r][0], 1, rt_s[r], inv_dt);
+                ry = realtime_term(a, ry, rt_l[r][1], 2, rt_s[r], inv_dt);
             }
-            if ((nfx + tfy) & 1) rx = -rx;
-            if ((nfy + tfx) & 1) ry = -ry;
-            sm.rt[0][k] = rx;
-            sm.rt[1][k] = ry;
+            sm.rt[0][k] = rt_f[r] & 1 ? -rx : rx;
+            sm.rt[1][k] = rt_f[r] & 2 ? -ry : ry;
         }
     }
     __syncthreads();
@@ -298,7 +387,10 @@ stage_kernel(const SweepArgs<T> a) {
     // the last bit, formed with fewer FP64 instructions.
     const T klim = T(a.limiter_k);
     const T kp = (a.gradp == kGradSuperbee || a.gradp == kGradSplitSuperbee) ? T(2) : T(1);
-    for (int k = tid; k < GW * GH; k += NT) {
+    const int grp = GR == 2 ? tid / NTG : 0, tg = tid - grp * NTG;
+    constexpr int R0 = GR == 2 ? TY / 2 + 2 : GH;      // ring rows the first group's faces need
+    if (GR == 2 && grp == 1) bar_sync(3, NT);          // the first group's slopes first
+    for (int k = grp * (R0 * GW) + tg; k < (GR == 2 && grp == 0 ? R0 * GW : GW * GH); k += NTG) {
         const int li = k % GW, lj = k / GW;            // ring coords (cell li-1, lj-1)
         const int c = (lj + 1) * RW + (li + 1);
         const int e = c + 1, wv = c - 1, nn = c + RW, ss = c - RW;
@@ -328,11 +420,14 @@ stage_kernel(const SweepArgs<T> a) {
             const T rho_g = wall_ghost_sign<T>(gi, gj, nx, ny, a.bc) < T(0) ? -rho : rho;
             const T rtx = need_rt ? sm.rt[0][k] : T(0);
             const T rty = need_rt ? sm.rt[1][k] : T(0);
-            const T ru = rho * u, rv = rho * v, uv = u * v;
-            spx = a.dx * fma(rho_g, a.gx, -rtx) - (u * u * srx + T(2) * ru * sux) -
-                  a.dx_over_dy * (uv * sry + ru * svy + rv * suy);
-            spy = a.dy * fma(rho_g, a.gy, -rty) - (v * v * sry + T(2) * rv * svy) -
-                  a.dy_over_dx * (uv * srx + rv * sux + ru * svx);
+            // d(rho u u) = u A + rho u du with A = d(rho u) along x, d(rho u v) = v A + rho u dv, and so on: 20 FP64
+            // instructions in place of 27 term by term
+            const T ru = rho * u, rv = rho * v;
+            const T A = fma(rho, sux, u * srx), B = fma(rho, svy, v * sry);
+            const T xx = fma(u, A, ru * sux), xy = fma(u, B, rv * suy);
+            const T yy = fma(v, B, rv * svy), yx = fma(v, A, ru * svx);
+            spx = fma(-a.dx_over_dy, xy, fma(a.dx, fma(rho_g, a.gx, -rtx), -xx));
+            spy = fma(-a.dy_over_dx, yx, fma(a.dy, fma(rho_g, a.gy, -rty), -yy));
         } else if (a.gradp == kGradSplitMinmod || a.gradp == kGradSplitSuperbee) {
             // Qian et al. split (Sec. 2.3.2): limit the kinematic part of the
             // one-sided pressure differences, add the cell's hydrostatic
@@ -351,26 +446,32 @@ stage_kernel(const SweepArgs<T> a) {
         sm.gx[0][k] = srx; sm.gx[1][k] = sux; sm.gx[2][k] = svx; sm.gx[3][k] = spx;
         sm.gy[0][k] = sry; sm.gy[1][k] = suy; sm.gy[2][k] = svy; sm.gy[3][k] = spy;
     }
-    __syncthreads();
+    if (GR == 2) {
+        if (grp == 0) bar_arrive(3, NT);
+        bar_sync(1 + grp, NTG);
+    } else {
+        __syncthreads();
+    }
 
     // ---- 3. face states and Osher fluxes ----
-    // The faces are dealt out so that the four SM sub-partitions get equal
-    // numbers of warp-passes (the FP64 pipe, not issue, bounds this loop, and
-    // a pass costs the same with idle lanes).  The warps of a CTA sit on
-    // contiguous slots, so warps w and w + 4 share a sub-partition; group
-    // w mod 4 takes faces [32 P g, 32 P (g + 1)), P = ceil(F / 128), in
-    // passes of 32 shared round-robin by its warps.  The plain strided loop
-    // gives the first warps an extra pass when the warp count is not a
-    // multiple of 4 (32x14 tiles: 9 warp-passes on two sub-partitions
-    // against 8 here).
-    constexpr int NF = S::NXF + S::NYF, NW = NT / 32, FP = (NF + 127) / 128;
-    static_assert(NW >= 4, "face schedule needs four warps");
-    const int fw = tid >> 5, fgrp = fw & 3;
-    const int fwarps = (NW - fgrp + 3) >> 2;
-    const int fbeg = fgrp * 32 * FP, fend = min(NF, fbeg + 32 * FP);
-    for (int fq = fw >> 2; fbeg + 32 * fq < fend; fq += fwarps) {
-        const int k = fbeg + 32 * fq + (tid & 31);
-        if (k >= fend) continue;
+    // A group's faces are dealt out so that the four SM sub-partitions get
+    // equal numbers of warp-passes (a pass costs the same with idle lanes).
+    // The warps of a CTA sit on contiguous slots, so warps w and w + 4 share a
+    // sub-partition; its share, faces [32 P s, 32 P (s + 1)) of the group's F,
+    // P = ceil(F / 128), goes to its warps of the group in passes of 32, round-robin.
+    constexpr int NWG = NTG / 32, XG = S::NXF / GR;   // warps and x-faces of a group
+    static_assert(NWG >= 4, "face schedule needs four warps");
+    const int yf0 = GR == 2 && grp == 1 ? (TY / 2 + 1) * TX : 0;                    // the group's first y-face
+    const int yfn = GR == 2 ? (grp == 0 ? (TY / 2 + 1) * TX : (TY / 2) * TX) : S::NYF;   // and their number
+    const int nf = XG + yfn, fp = (nf + 127) / 128;
+    const int fw = tid >> 5, sub = fw & 3;
+    const int w0 = grp * NWG + ((sub - grp * NWG) & 3);            // the sub-partition's first warp of the group
+    const int fwarps = (grp * NWG + NWG - w0 + 3) >> 2;
+    const int fbeg = sub * 32 * fp, fend = min(nf, fbeg + 32 * fp);
+    for (int fq = (fw - w0) >> 2; fbeg + 32 * fq < fend; fq += fwarps) {
+        const int kf = fbeg + 32 * fq + (tid & 31);
+        if (kf >= fend) continue;
+        const int k = kf < XG ? grp * XG + kf : S::NXF + yf0 + (kf - XG);
         const bool isx = k < S::NXF;
         // face states: density, normal and tangential velocity (rotation,
         // Alg. 2: (u, v) on x-faces, (v, u) on y-faces), pressure
@@ -396,13 +497,20 @@ stage_kernel(const SweepArgs<T> a) {
             pL = fma(T(0.5), sm.gy[3][ga], sm.w[3][ca]); pR = fma(T(-0.5), sm.gy[3][gb], sm.w[3][cb]);
             fo = kk;
         }
-        // one flux call for both kinds: no divergence where a warp holds both
-        // (2F: the divergence below takes the 1/2)
+        // one flux call for both kinds: no divergence where a warp holds both.
+        // Fluxes are stored as F/dx or F/dy (formed as 2F times 1/(2 dx)), the
+        // pressure row times beta, so that the divergence is sums only.
         T F[4];
-        if (RS == kOsher && fixed_flux_ok(rL, nL, tL, pL, rR, nR, tR, pR))
-            osher_flux_fixed(rL, nL, tL, pL, rR, nR, tR, pR, a.fbeta, F);
-        else
+        if (RS == kOsher && a.fixed && fixed_flux_ok(rL, nL, tL, pL, rR, nR, tR, pR)) {
+            osher_flux_fixed(rL, nL, tL, pL, rR, nR, tR, pR, a.fbeta, isx ? a.fhx : a.fhy, isx ? a.fphx : a.fphy, F);
+        } else {
             riemann_flux<RS, T, true>(rL, nL, tL, pL, rR, nR, tR, pR, a.beta, a.inv_beta, F);
+            const T h = isx ? a.hidx : a.hidy;
+            F[0] *= h;
+            F[1] *= h;
+            F[2] *= h;
+            F[3] *= isx ? a.phidx : a.phidy;
+        }
         T *fd = isx ? &sm.fx[0][fo] : &sm.fy[0][fo];
         const int fs = isx ? S::NXF : S::NYF;
         fd[0] = F[0];
@@ -410,23 +518,32 @@ stage_kernel(const SweepArgs<T> a) {
         fd[2 * fs] = isx ? F[2] : F[1];
         fd[3 * fs] = F[3];
     }
-    __syncthreads();
+    if (GR == 2) {
+        // the second group's lowest cells take the y-faces between the groups
+        if (grp == 0) {
+            bar_arrive(4, NT);
+            bar_sync(1, NTG);
+        } else {
+            bar_sync(4, NT);
+        }
+    } else {
+        __syncthreads();
+    }
 
     // ---- 4. divergence + sources + point-implicit stage update ----
-    const int li = tid % TX, lj = tid / TX;
+    constexpr int CG = TX * TY / GR;   // cells of a group
+    const int cell = grp * CG + tg;
+    const int li = cell % TX, lj = cell / TX;
     const int gi = x0 + li, gj = y0 + lj;
-    const bool inside = (gi < nx) && (gj < ny);
+    const bool inside = (tg < CG) && (gi < nx) && (gj < ny);
     double sq[4] = {0.0, 0.0, 0.0, 0.0};
     if (inside) {
         const size_t g = (size_t)gj * nx + gi;
         const int fw = lj * (TX + 1) + li, fe = fw + 1;
         const int fs = lj * TX + li, fn = fs + TX;
-        // fluxes are stored doubled: (2Fe - 2Fw) (1/(2 dx)) is (Fe - Fw)/dx exactly
-        const T hidx = T(0.5) * a.inv_dx, hidy = T(0.5) * a.inv_dy;
         T div[4];
 #pragma unroll
-        for (int f = 0; f < 4; ++f)
-            div[f] = (sm.fx[f][fe] - sm.fx[f][fw]) * hidx + (sm.fy[f][fn] - sm.fy[f][fs]) * hidy;
+        for (int f = 0; f < 4; ++f) div[f] = (sm.fx[f][fe] - sm.fx[f][fw]) + (sm.fy[f][fn] - sm.fy[f][fs]);
         const T r0 = q0[0][g], m0 = q0[1][g], n0 = q0[2][g], p0 = q0[3][g];
         // At stage 1 the input Q^{s-1} is Q^{m} itself, so the cell's W (never
         // a folded ghost here) holds the 1/rho, u and v of Q^{m}, and the ring
@@ -457,13 +574,16 @@ stage_kernel(const SweepArgs<T> a) {
             }
         }
         const T b0 = -div[0] - rt0;
-        const T b1 = -div[1] - rt1 + r0 * a.gx;
-        const T b2 = -div[2] - rt2 + r0 * a.gy;
-        const T b3 = -div[3];
-        // pseudo-time step from Q^{m} (Sec. 2.2.3)
-        T dtau;
+        T b1 = -div[1] - rt1;
+        T b2 = -div[2] - rt2;
+        if (a.gx != T(0)) b1 = fma(r0, a.gx, b1);
+        if (a.gy != T(0)) b2 = fma(r0, a.gy, b2);
+        const T b3 = -div[3];   // in pressure units
+        // pseudo-time step from Q^{m} (Sec. 2.2.3), kept as 1/dtau: Eq. point_implicit's
+        // alpha dtau / (1 + B0 alpha dtau/dt) is 1 / (1/(alpha dtau) + B0/dt), one reciprocal
+        T idt;
         if (a.local_dtau && reuse_now) {
-            dtau = a.aux[0][g];
+            idt = a.aux[0][g];
         } else if (a.local_dtau) {
             T ir, u, v;
             if (from_tile) {
@@ -475,42 +595,40 @@ stage_kernel(const SweepArgs<T> a) {
                 u = m0 * ir;
                 v = n0 * ir;
             }
-            const T fb = T(4) * a.beta * ir;
-            // square roots as x / sqrt(x) and quotients as products with a
-            // rounded reciprocal: a few ulps, far inside the 1e-11 bar
+            const T fb = (T(4) * a.beta) * ir;
             T cx, cy, unused;
-            Ar<T>::sqrt_rsqrt(u * u + fb, cx, unused);
-            Ar<T>::sqrt_rsqrt(v * v + fb, cy, unused);
-            const T den = T(0.5) * (fabs(u) + cx) * a.dy + T(0.5) * (fabs(v) + cy) * a.dx;
-            dtau = a.cfl_area * Ar<T>::rcp(den);
-            if (a.reuse) a.aux[0][g] = dtau;
+            Ar<T>::sqrt_rsqrt(fma(u, u, fb), cx, unused);
+            Ar<T>::sqrt_rsqrt(fma(v, v, fb), cy, unused);
+            idt = fma(fabs(u) + cx, a.half_dy, (fabs(v) + cy) * a.half_dx) * a.inv_cfl_area;
+            if (a.reuse) a.aux[0][g] = idt;
         } else {
-            dtau = T(global_dtau(ctl));
+            idt = Ar<T>::rcp(T(global_dtau(ctl)));
         }
-        const T api = T(1) + a.B[0] * a.alpha * dtau * inv_dt;   // Eq. point_implicit
-        const T coef = (a.alpha * dtau) * Ar<T>::rcp(api);
-        const T coef_p = a.alpha_pi_p_row ? coef : a.alpha * dtau;
-        qout[0][g] = r0 + coef * b0;
-        qout[1][g] = m0 + coef * b1;
-        qout[2][g] = n0 + coef * b2;
-        qout[3][g] = p0 + a.beta * coef_p * b3;
+        const T coef = Ar<T>::rcp(fma(idt, a.inv_alpha, a.B[0] * inv_dt));
+        const T coef_p = a.alpha_pi_p_row ? coef : Ar<T>::rcp(idt * a.inv_alpha);
+        qout[0][g] = fma(coef, b0, r0);
+        qout[1][g] = fma(coef, b1, m0);
+        qout[2][g] = fma(coef, b2, n0);
+        qout[3][g] = fma(coef_p, b3, p0);
         if (a.stage == 1) {
-            const double pb = double(a.beta) * double(b3);
             sq[0] = double(b0) * double(b0);
             sq[1] = double(b1) * double(b1);
             sq[2] = double(b2) * double(b2);
-            sq[3] = pb * pb;
+            sq[3] = double(b3) * double(b3);
         }
     }
     if (a.stage == 1) {
-        // deterministic block reduction of the squared bracket (FP64)
+        // deterministic block reduction of the squared bracket (FP64): the
+        // first two exchanges leave each lane one of the four sums, so a warp
+        // spends 6 additions instead of 20
+        const int lane = tid & 31;
+        const bool up16 = lane & 16, up8 = lane & 8;
+        double v0 = (up16 ? sq[2] : sq[0]) + __shfl_xor_sync(0xffffffffu, up16 ? sq[0] : sq[2], 16);
+        const double v1 = (up16 ? sq[3] : sq[1]) + __shfl_xor_sync(0xffffffffu, up16 ? sq[1] : sq[3], 16);
+        v0 = (up8 ? v1 : v0) + __shfl_xor_sync(0xffffffffu, up8 ? v0 : v1, 8);
 #pragma unroll
-        for (int f = 0; f < 4; ++f) {
-            double v = sq[f];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-            if ((tid & 31) == 0) sm.red[f][tid >> 5] = v;
-        }
+        for (int o = 4; o > 0; o >>= 1) v0 += __shfl_xor_sync(0xffffffffu, v0, o);
+        if ((lane & 7) == 0) sm.red[lane >> 3][tid >> 5] = v0;   // field 2 (lane/16) + (lane/8 mod 2)
         __syncthreads();
         if (tid < 4) {
             double s = 0.0;

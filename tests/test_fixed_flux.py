@@ -19,7 +19,8 @@ WRAPPER = r'''
 #include "ac_fixed_flux.cuh"
 extern "C" int fixed_flux(const double *s, double beta, double *F) {
     if (!acgb::fixed_flux_ok(s[0], s[1], s[2], s[3], s[4], s[5], s[6], s[7])) return 0;
-    acgb::osher_flux_fixed(s[0], s[1], s[2], s[3], s[4], s[5], s[6], s[7], acgb::make_fixed_beta(beta), F);
+    acgb::osher_flux_fixed(s[0], s[1], s[2], s[3], s[4], s[5], s[6], s[7], acgb::make_fixed_beta(beta),
+                           acgb::make_fixed_scale(1.0), acgb::make_fixed_scale(1.0), F);
     return 1;
 }
 extern "C" void iterations(unsigned long long x, unsigned long long *out) {
@@ -110,11 +111,19 @@ def test_mirrored_states_pass_no_mass_and_rest_stays_at_rest(lib):
         assert flux(lib, [r, 0.0, 0.0, p, 1.0, 0.0, 0.0, p], 4e5) == [0.0, 2.0 * p, 0.0, 0.0]
 
 
+def test_zeros_and_subnormals_count_as_zero(lib):
+    """Exact zeros give exact zeros, and a subnormal velocity what a zero one gives."""
+    for tiny in (0.0, -0.0, 5e-324, -1e-310):
+        assert flux(lib, [3.0, tiny, tiny, 0.0, 3.0, tiny, tiny, 0.0], 10.0) == [0.0, 0.0, 0.0, 0.0]
+        assert flux(lib, [3.0, tiny, 0.0, 1.5, 2.0, 0.25, tiny, 2.5], 10.0) == flux(
+            lib, [3.0, 0.0, 0.0, 1.5, 2.0, 0.25, 0.0, 2.5], 10.0)
+
+
 def test_refuses_what_it_cannot_represent(lib):
     good = [1.0, 0.5, 0.1, 2.0, 3.0, -0.5, 0.0, 1.0]
     assert flux(lib, good, 10.0) is not None
     for k in range(8):
-        for bad in (np.inf, -np.inf, np.nan) + ((0.0, -1.0, 5e-324) if k in (0, 4) else ()):
+        for bad in (np.inf, -np.inf, np.nan, 1e80, -1e80) + ((0.0, -1.0, 5e-324, 1e-80) if k in (0, 4) else ()):
             s = list(good)
             s[k] = bad
             assert flux(lib, s, 10.0) is None, (k, bad)
