@@ -30,6 +30,7 @@
 #include "ac_internal.h"
 #include "ac_kernels_mixed.cuh"
 #include "ac_mixed_host.h"
+#include "ac_state.cuh"
 
 using namespace acgb;
 
@@ -112,6 +113,7 @@ struct ac_ctx {
     double stage_ms;
     long long stage_launches;
     unsigned long long *dt_word;   // device result of ac_realtime_dt
+    int *bad;                      // device result of a new state's check
     bool pdl;             // launch the loop's kernels with programmatic dependencies
     int nhist;            // older real-time levels held (0..2) before the next step
     int order_now;        // backward-difference order of the current step
@@ -129,7 +131,9 @@ struct Backend {
     virtual int tune(ac_ctx *c, cudaStream_t s) { (void)c; (void)s; return AC_OK; }
     virtual int alloc(ac_ctx *c) = 0;
     virtual void release() = 0;
-    virtual int set_state(ac_ctx *c, const double *const f[4]) = 0;
+    // copies, checks (densities within [lo, hi]) and takes a new state; `buf` receives the buffer that holds it and
+    // `bad` whether the fields were refused (the old state stays)
+    virtual int set_state(ac_ctx *c, const double *const f[4], double lo, double hi, int &buf, int &bad) = 0;
     virtual int get_state(const ac_ctx *c, double *const out[4]) = 0;
     virtual int get_history(const ac_ctx *c, int k, double *const out[3]) = 0;
     virtual int set_history(ac_ctx *c, int k, const double *const in[3]) = 0;
@@ -337,12 +341,16 @@ struct F64Backend : Backend {
         for (int f = 0; f < 4; ++f) { cudaFree(lev[f]); cudaFree(aux[f]); }
         for (int f = 0; f < 3; ++f) { cudaFree(lev1[f]); cudaFree(lev2[f]); }
     }
-    int set_state(ac_ctx *c, const double *const f[4]) override {
-        const size_t bytes = c->N * sizeof(double);
-        for (int k = 0; k < 4; ++k) {
-            CK(cudaMemcpyAsync(buf[0][k], f[k], bytes, cudaMemcpyHostToDevice, c->stream));
-            CK(cudaMemcpyAsync(lev[k], f[k], bytes, cudaMemcpyHostToDevice, c->stream));
-        }
+    // into a scratch buffer, which becomes the current one if its fields are good
+    int set_state(ac_ctx *c, const double *const f[4], double lo, double hi, int &nbuf, int &bad) override {
+        nbuf = (c->cur_host + 1) % 3;
+        const Staged st{{buf[nbuf][0], buf[nbuf][1], buf[nbuf][2], buf[nbuf][3]}}, lv{{lev[0], lev[1], lev[2], lev[3]}};
+        const int blocks = grid_stride_blocks(c->N);
+        CK(stage_fields(f, st, c->N, lo, hi, c->bad, blocks, c->stream));
+        level_from_fields_kernel<<<blocks, 256, 0, c->stream>>>(st, lv, c->N, c->bad);
+        CK(cudaGetLastError());
+        CK(cudaMemcpyAsync(&bad, c->bad, sizeof bad, cudaMemcpyDeviceToHost, c->stream));
+        CK(cudaStreamSynchronize(c->stream));
         return AC_OK;
     }
     int get_state(const ac_ctx *c, double *const out[4]) override {
@@ -669,44 +677,34 @@ struct MixedBackend : Backend {
         cudaFree(dtau);
         for (int f = 0; f < 3; ++f) { cudaFree(D1[f]); cudaFree(D2[f]); }
     }
-    int set_state(ac_ctx *c, const double *const f[4]) override {
-        const size_t N = c->N;
-        for (int q = 0; q < 3; ++q) {
-            if (D1[q]) CK(cudaMemsetAsync(D1[q], 0, N * sizeof(float), c->stream));
-            if (D2[q]) CK(cudaMemsetAsync(D2[q], 0, N * sizeof(float), c->stream));
-        }
-        MixedReference ref;
-        build_mixed_reference(c->grid.nx, c->grid.ny, c->dy, c->grid.gy, use_ref, plevel, f, ref);
+    // staged in the two scratch buffers; the current one keeps its place
+    Staged staged(const ac_ctx *c) const {
+        return staged_in(d[(c->cur_host + 1) % 3], d[(c->cur_host + 2) % 3], c->N);
+    }
+    int set_state(ac_ctx *c, const double *const f[4], double lo, double hi, int &nbuf, int &bad) override {
+        nbuf = c->cur_host;
+        const Staged st = staged(c);
+        const int blocks = grid_stride_blocks(c->N);
         cudaStream_t s = c->stream;
-        const size_t fb = N * sizeof(float), db = N * sizeof(double);
-        // the two per-cell records: (Q^n in FP32, rho_ref) and (dQ = 0, dp = 0 or p)
-        std::vector<float4> hq(N), hd(N);
-        for (size_t q = 0; q < N; ++q) {
-            hq[q] = make_float4(float(f[0][q]), float(f[1][q]), float(f[2][q]), ref.rho_ref[q]);
-            hd[q] = make_float4(0.0f, 0.0f, 0.0f, ref.p_record[q]);
-        }
-        for (int k = 0; k < 3; ++k) CK(cudaMemcpyAsync(q64[k], f[k], db, cudaMemcpyHostToDevice, s));
-        CK(cudaMemcpyAsync(q64[3], ref.p_level.data(), db, cudaMemcpyHostToDevice, s));
-        if (pref64) CK(cudaMemcpyAsync(pref64, ref.p_ref.data(), db, cudaMemcpyHostToDevice, s));
-        CK(cudaMemcpyAsync(qn, hq.data(), N * sizeof(float4), cudaMemcpyHostToDevice, s));
-        CK(cudaMemcpyAsync(d[0], hd.data(), N * sizeof(float4), cudaMemcpyHostToDevice, s));
-        CK(cudaMemcpyAsync(lev_p, ref.p_record.data(), fb, cudaMemcpyHostToDevice, s));
+        CK(stage_fields(f, st, c->N, lo, hi, c->bad, blocks, s));
+        CK(mixed_from_fields(st, args(c, 0), d[nbuf], use_ref, c->grid.gy, c->dy, c->bad, blocks, s));
+        CK(cudaMemcpyAsync(&bad, c->bad, sizeof bad, cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
+        if (bad) return AC_OK;
+        for (int q = 0; q < 3; ++q) {
+            if (D1[q]) CK(cudaMemsetAsync(D1[q], 0, c->N * sizeof(float), s));
+            if (D2[q]) CK(cudaMemsetAsync(D2[q], 0, c->N * sizeof(float), s));
+        }
         return AC_OK;
     }
     int get_state(const ac_ctx *c, double *const out[4]) override {
-        const size_t N = c->N;
-        std::vector<float4> h(N);
-        const int cur = c->cur_host;
-        CK(cudaMemcpyAsync(h.data(), d[cur], N * sizeof(float4), cudaMemcpyDeviceToHost, c->stream));
+        const Staged st = staged(c);
+        mixed_to_fields_kernel<<<grid_stride_blocks(c->N), 256, 0, c->stream>>>(args(c, 0), d[c->cur_host], st, c->N);
+        CK(cudaGetLastError());
         for (int k = 0; k < 4; ++k)
-            if (out[k]) CK(cudaMemcpyAsync(out[k], q64[k], N * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+            if (out[k])
+                CK(cudaMemcpyAsync(out[k], st.f[k], c->N * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
         CK(cudaStreamSynchronize(c->stream));
-        // state = FP64 level + FP32 increment
-        if (out[0]) for (size_t q = 0; q < N; ++q) out[0][q] += double(h[q].x);
-        if (out[1]) for (size_t q = 0; q < N; ++q) out[1][q] += double(h[q].y);
-        if (out[2]) for (size_t q = 0; q < N; ++q) out[2][q] += double(h[q].z);
-        if (out[3]) for (size_t q = 0; q < N; ++q) out[3][q] += double(h[q].w);
         return AC_OK;
     }
     // Between steps, history 1 is the FP64 level q64 and history 2 is
@@ -998,6 +996,7 @@ int ac_create(const ac_grid *grid, const ac_fluids *fluids, double beta, const a
     CKC(cudaMalloc(&c->partials, max_tiles(grid->nx, grid->ny) * 4 * sizeof(double)));
     CKC(cudaMalloc(&c->ctl, sizeof(Ctl)));
     CKC(cudaMalloc(&c->dt_word, sizeof(unsigned long long)));
+    CKC(cudaMalloc(&c->bad, sizeof(int)));
     CKC(cudaMallocHost(&c->hctl, sizeof(Ctl)));
     CKC(cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking));
     for (int k = 0; k < 5; ++k) CKC(cudaEventCreate(&c->ev[k]));
@@ -1022,6 +1021,7 @@ void ac_destroy(ac_ctx *c) {
     cudaFree(c->partials);
     cudaFree(c->ctl);
     cudaFree(c->dt_word);
+    cudaFree(c->bad);
     if (c->hctl) cudaFreeHost(c->hctl);
     delete c;
 }
@@ -1032,9 +1032,8 @@ int ac_set_stream(ac_ctx *c, void *stream) {
     return AC_OK;
 }
 
-int ac_set_state(ac_ctx *c, const double *rho, const double *rhou, const double *rhov, const double *p) {
-    g_err.clear();
-    if (!c) return fail(AC_ERR_ARG, "ctx is NULL");
+// Why the device refused a new state: the first field and cell at fault, in the fields' order.
+static int refused_state(const ac_ctx *c, const double *rho, const double *rhou, const double *rhov, const double *p) {
     int rc;
     if ((rc = check_host_field(rho, c->N, true, "rho")) != AC_OK) return rc;
     if ((rc = check_host_field(rhou, c->N, false, "rhou")) != AC_OK) return rc;
@@ -1045,15 +1044,26 @@ int ac_set_state(ac_ctx *c, const double *rho, const double *rhou, const double 
             if (rho[k] < 0.5 * c->fluids.rho_light || rho[k] > 2.0 * c->fluids.rho_heavy)
                 return fail(AC_ERR_ARG, "rho[%zu] = %g lies outside [rho_light/2, 2 rho_heavy]", k, rho[k]);
     }
+    return fail(AC_ERR_ARG, "the fields changed during the call");
+}
+
+int ac_set_state(ac_ctx *c, const double *rho, const double *rhou, const double *rhov, const double *p) {
+    g_err.clear();
+    if (!c) return fail(AC_ERR_ARG, "ctx is NULL");
     const double *src[4] = {rho, rhou, rhov, p};
-    CK(cudaStreamSynchronize(c->stream));
-    if ((rc = c->be->set_state(c, src)) != AC_OK) return rc;
-    c->hctl->cur = 0;
+    for (int k = 0; k < 4; ++k)
+        if (!src[k]) return refused_state(c, rho, rhou, rhov, p);   // (an earlier field's fault comes first)
+    const double lo = c->has_fluids ? 0.5 * c->fluids.rho_light : 0.0;
+    const double hi = c->has_fluids ? 2.0 * c->fluids.rho_heavy : INFINITY;
+    int rc, buf = 0, bad = 0;
+    if ((rc = c->be->set_state(c, src, lo, hi, buf, bad)) != AC_OK) return rc;
+    if (bad) return refused_state(c, rho, rhou, rhov, p);
+    c->hctl->cur = buf;
     c->hctl->done = 1;
     c->hctl->iter = 0;
     CK(cudaMemcpyAsync(c->ctl, c->hctl, sizeof(Ctl), cudaMemcpyHostToDevice, c->stream));
     CK(cudaStreamSynchronize(c->stream));
-    c->cur_host = 0;
+    c->cur_host = buf;
     c->nhist = 0;
     c->has_state = true;
     return AC_OK;

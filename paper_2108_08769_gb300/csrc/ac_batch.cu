@@ -27,6 +27,7 @@
 #include "ac_internal.h"
 #include "ac_kernels_mixed.cuh"
 #include "ac_mixed_host.h"
+#include "ac_state.cuh"
 
 using namespace acgb;
 
@@ -348,6 +349,7 @@ struct ac_batch {
     double *partials;
     Ctl *ctl;
     BatchSync *sync;
+    int *bad;                           // a new state's check
     BatchTank *tanks_dev;
     int *tile_map;                      // per variant: flattened tile -> tank
     double *dt_dev;
@@ -577,6 +579,7 @@ void ac_batch_destroy(ac_batch *b) {
     cudaFree(b->partials);
     cudaFree(b->ctl);
     cudaFree(b->sync);
+    cudaFree(b->bad);
     cudaFree(b->tanks_dev);
     cudaFree(b->tile_map);
     cudaFree(b->dt_dev);
@@ -668,6 +671,7 @@ int ac_batch_create(int n, const ac_grid *grids, const double *beta, const ac_bc
     CKB(cudaMalloc(&b->tile_map, max_tiles * sizeof(int)));
     CKB(cudaMalloc(&b->ctl, n * sizeof(Ctl)));
     CKB(cudaMalloc(&b->sync, sizeof(BatchSync)));
+    CKB(cudaMalloc(&b->bad, sizeof(int)));
     CKB(cudaMalloc(&b->tanks_dev, n * sizeof(BatchTank)));
     CKB(cudaMalloc(&b->dt_dev, n * sizeof(double)));
     CKB(cudaMallocHost(&b->hctl, n * sizeof(Ctl)));
@@ -754,40 +758,37 @@ int ac_batch_set_state(ac_batch *b, int k, const double *rho, const double *rhou
     if (!b) return fail(AC_ERR_ARG, "batch is NULL");
     if (k < 0 || k >= b->n) return fail(AC_ERR_ARG, "tank index %d out of range", k);
     const size_t N = (size_t)b->grids[k].nx * b->grids[k].ny;
-    int rc;
-    if ((rc = check_field(rho, N, true, "rho")) != AC_OK) return rc;
-    if ((rc = check_field(rhou, N, false, "rhou")) != AC_OK) return rc;
-    if ((rc = check_field(rhov, N, false, "rhov")) != AC_OK) return rc;
-    if ((rc = check_field(p, N, false, "p")) != AC_OK) return rc;
     const double *f[4] = {rho, rhou, rhov, p};
+    auto refused = [&] {   // the first field and cell at fault
+        int rc;
+        if ((rc = check_field(rho, N, true, "rho")) != AC_OK) return rc;
+        if ((rc = check_field(rhou, N, false, "rhou")) != AC_OK) return rc;
+        if ((rc = check_field(rhov, N, false, "rhov")) != AC_OK) return rc;
+        if ((rc = check_field(p, N, false, "p")) != AC_OK) return rc;
+        return fail(AC_ERR_ARG, "the fields changed during the call");
+    };
+    for (int q = 0; q < 4; ++q)
+        if (!f[q]) return refused();   // (an earlier field's fault comes first)
     const ac_grid &g = b->grids[k];
-    MixedReference ref;
-    build_mixed_reference(g.nx, g.ny, g.ly / g.ny, g.gy, b->use_ref[k] != 0, b->plevel, f, ref);
     cudaStream_t s = b->stream;
+    // staged in the tank's part of the two pools that do not hold its state; its buffer keeps its place
+    const int cur = b->hctl[k].cur, blocks = (int)std::min<size_t>((N + 255) / 256, 152 * 8);
+    const size_t o = b->off[k], fb = N * sizeof(float);
+    const Staged st = staged_in(b->d[(cur + 1) % 3] + o, b->d[(cur + 2) % 3] + o, N);
+    int bad = 0;
+    CK(stage_fields(f, st, N, 0.0, INFINITY, b->bad, blocks, s));
+    CK(mixed_from_fields(st, b->tanks_host[k].a, b->d[cur] + o, b->use_ref[k] != 0, g.gy, g.ly / g.ny, b->bad, blocks,
+                         s));
+    CK(cudaMemcpyAsync(&bad, b->bad, sizeof bad, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
-    // the tank's control block: buffer 0 holds its state from now on
-    Ctl hc;
-    CK(cudaMemcpy(&hc, b->ctl + k, sizeof(Ctl), cudaMemcpyDeviceToHost));
-    hc.cur = 0;
-    hc.done = 1;
-    hc.iter = 0;
-    const size_t o = b->off[k], fb = N * sizeof(float), db = N * sizeof(double);
-    // the two per-cell records: (Q^n in FP32, rho_ref) and (dQ = 0, dp = 0 or p)
-    std::vector<float4> hq(N), hd(N);
-    for (size_t i = 0; i < N; ++i) {
-        hq[i] = make_float4(float(f[0][i]), float(f[1][i]), float(f[2][i]), ref.rho_ref[i]);
-        hd[i] = make_float4(0.0f, 0.0f, 0.0f, ref.p_record[i]);
-    }
-    for (int q = 0; q < 3; ++q) CK(cudaMemcpyAsync(b->q64[q] + o, f[q], db, cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(b->q64[3] + o, ref.p_level.data(), db, cudaMemcpyHostToDevice, s));
-    if (b->use_ref[k]) CK(cudaMemcpyAsync(b->pref64 + o, ref.p_ref.data(), db, cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(b->qn + o, hq.data(), N * sizeof(float4), cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(b->d[0] + o, hd.data(), N * sizeof(float4), cudaMemcpyHostToDevice, s));
+    if (bad) return refused();
     for (int q = 0; q < 3; ++q) {
         if (b->D1[q]) CK(cudaMemsetAsync(b->D1[q] + o, 0, fb, s));
         if (b->D2[q]) CK(cudaMemsetAsync(b->D2[q] + o, 0, fb, s));
     }
-    CK(cudaMemcpyAsync(b->lev_p + o, ref.p_record.data(), fb, cudaMemcpyHostToDevice, s));
+    Ctl hc = b->hctl[k];
+    hc.done = 1;
+    hc.iter = 0;
     CK(cudaMemcpyAsync(b->ctl + k, &hc, sizeof(Ctl), cudaMemcpyHostToDevice, s));
     CK(cudaStreamSynchronize(s));
     b->hctl[k] = hc;
@@ -800,18 +801,14 @@ int ac_batch_get_state(const ac_batch *b, int k, double *rho, double *rhou, doub
     if (!b) return fail(AC_ERR_ARG, "batch is NULL");
     if (k < 0 || k >= b->n) return fail(AC_ERR_ARG, "tank index %d out of range", k);
     const size_t N = (size_t)b->grids[k].nx * b->grids[k].ny, o = b->off[k];
-    const int cur = b->hctl[k].cur;
+    const int cur = b->hctl[k].cur, blocks = (int)std::min<size_t>((N + 255) / 256, 152 * 8);
     double *out[4] = {rho, rhou, rhov, p};
-    std::vector<float4> h(N);
-    CK(cudaMemcpyAsync(h.data(), b->d[cur] + o, N * sizeof(float4), cudaMemcpyDeviceToHost, b->stream));
+    const Staged st = staged_in(b->d[(cur + 1) % 3] + o, b->d[(cur + 2) % 3] + o, N);
+    mixed_to_fields_kernel<<<blocks, 256, 0, b->stream>>>(b->tanks_host[k].a, b->d[cur] + o, st, N);
+    CK(cudaGetLastError());
     for (int q = 0; q < 4; ++q)
-        if (out[q]) CK(cudaMemcpyAsync(out[q], b->q64[q] + o, N * sizeof(double), cudaMemcpyDeviceToHost, b->stream));
+        if (out[q]) CK(cudaMemcpyAsync(out[q], st.f[q], N * sizeof(double), cudaMemcpyDeviceToHost, b->stream));
     CK(cudaStreamSynchronize(b->stream));
-    // state = FP64 level + FP32 increment
-    if (rho) for (size_t i = 0; i < N; ++i) rho[i] += double(h[i].x);
-    if (rhou) for (size_t i = 0; i < N; ++i) rhou[i] += double(h[i].y);
-    if (rhov) for (size_t i = 0; i < N; ++i) rhov[i] += double(h[i].z);
-    if (p) for (size_t i = 0; i < N; ++i) p[i] += double(h[i].w);
     return AC_OK;
 }
 
