@@ -77,16 +77,18 @@ batch_stage_kernel(const BatchTank *__restrict__ tanks, const int *__restrict__ 
     const int k = tile_tank[blockIdx.x];
     if constexpr (CD) {
         const BatchTank &t = c_tanks[slot0 + k];
-        if (t.a.ctl->done) return;
+        const CtlHead<float> head = ctl_head<float>(t.a.ctl);
+        if (head.done) return;
         const int local = blockIdx.x - t.tile0;
         const int by = local / t.tiles_x, bx = local - by * t.tiles_x;
-        mixed_tile<TX, TY, NT, RS, BDF, PF>(t.a, stage, alpha, bx, by, t.a.partials + (size_t)local * 4, smem_raw);
+        mixed_tile<TX, TY, NT, RS, BDF, PF>(t.a, head, stage, alpha, bx, by, t.a.partials + (size_t)local * 4, smem_raw);
     } else {
         const BatchTank &t = tanks[k];
-        if (t.a.ctl->done) return;
+        const CtlHead<float> head = ctl_head<float>(t.a.ctl);
+        if (head.done) return;
         const int local = blockIdx.x - t.tile0;
         const int by = local / t.tiles_x, bx = local - by * t.tiles_x;
-        mixed_tile<TX, TY, NT, RS, BDF, PF>(t.a, stage, alpha, bx, by, t.a.partials + (size_t)local * 4, smem_raw);
+        mixed_tile<TX, TY, NT, RS, BDF, PF>(t.a, head, stage, alpha, bx, by, t.a.partials + (size_t)local * 4, smem_raw);
     }
 }
 
@@ -106,16 +108,18 @@ batch_sweep_kernel(const BatchTank *__restrict__ tanks, const int *__restrict__ 
     const int k = strip_tank[w];
     if constexpr (CD) {
         const BatchTank &t = c_tanks[slot0 + k];
-        if (t.a.ctl->done) return;
+        const CtlHead<float> head = ctl_head<float>(t.a.ctl);
+        if (head.done) return;
         const int local = w - t.tile0;
         const int sy = local / t.tiles_x, sx = local - sy * t.tiles_x;
-        mixed_strip<H, 1, SK>(t.a, stage, alpha, sx, sy, t.a.partials + (size_t)local * 4, ring);
+        mixed_strip<H, 1, SK>(t.a, head, stage, alpha, sx, sy, t.a.partials + (size_t)local * 4, ring);
     } else {
         const BatchTank &t = tanks[k];
-        if (t.a.ctl->done) return;
+        const CtlHead<float> head = ctl_head<float>(t.a.ctl);
+        if (head.done) return;
         const int local = w - t.tile0;
         const int sy = local / t.tiles_x, sx = local - sy * t.tiles_x;
-        mixed_strip<H, 1, SK>(t.a, stage, alpha, sx, sy, t.a.partials + (size_t)local * 4, ring);
+        mixed_strip<H, 1, SK>(t.a, head, stage, alpha, sx, sy, t.a.partials + (size_t)local * 4, ring);
     }
 }
 
@@ -196,30 +200,25 @@ batch_end_kernel(BatchTank *tanks, BatchSync *sync, int ntanks, unsigned long lo
     const BatchTank &t = tanks[blockIdx.x];
     Ctl *ctl = t.a.ctl;
     const bool was_done = ctl->done != 0;
-    double sums[4] = {0.0, 0.0, 0.0, 0.0};
-    if (!was_done) sum_partials_fixed(t.a.partials, t.ntiles, sums);
+    EndTest e;
+    double sum = 0.0;
+    if (!was_done) {
+        e.load(ctl);
+        sum = sum_partials_fixed(t.a.partials, t.ntiles);
+        if (tid < 4) e.judge(ctl, sum, 1.0 / ((double)t.a.nx * t.a.ny));
+    }
     if (tid == 0) {
         int active = 0;
         if (!was_done) {
-            const double inv_cells = 1.0 / ((double)t.a.nx * t.a.ny);
-            const int it = ctl->iter + 1;
-            ctl->iter = it;
-            bool finite = true, conv = true;
-            for (int f = 0; f < 4; ++f) {
-                const double R = sqrt(sums[f] * inv_cells);
-                ctl->R[f] = R;
-                if (it == 1) ctl->R0[f] = R;
-                if (!isfinite(R)) finite = false;
-                if (!(R <= fmax(ctl->tol * ctl->R0[f], ctl->abs_tol[f]))) conv = false;
-            }
-            ctl->cur = final_buffer(ctl->cur, t.a.s_max);
+            ctl->iter = e.it;
+            ctl->cur = final_buffer(e.cur, t.a.s_max);
             int done = 0;
-            if (!finite) { ctl->status = -3; done = 1; }
-            else if (!ctl->fixed && conv) { ctl->status = 0; done = 1; }
-            else if (it >= ctl->max_iters) { ctl->status = ctl->fixed ? 0 : 1; done = 1; }
+            if (!e.finite) { ctl->status = -3; done = 1; }
+            else if (!e.fixed && e.conv) { ctl->status = 0; done = 1; }
+            else if (e.it >= e.max_iters) { ctl->status = e.fixed ? 0 : 1; done = 1; }
             ctl->done = done;
             // pressure rebase after iterations 1, 2, 4, 8 (see mixed_rebase_shift)
-            ctl->rebase = (t.a.plevel && !done && rebase_after(it)) ? 1 : 0;
+            ctl->rebase = (t.a.plevel && !done && rebase_after(e.it)) ? 1 : 0;
             active = !done;
         }
         if (active) atomicAdd(&sync->still_active, 1u);
@@ -504,28 +503,54 @@ int tune(ac_batch *b, cudaStream_t s) {
     return build_tiles(b, int(std::min_element(tmin.begin(), tmin.end()) - tmin.begin()));
 }
 
-int enqueue_iteration(ac_batch *b, cudaStream_t s, unsigned long long cond, int use_cond, bool timed) {
+// One pseudo-iteration; rebase adds the kernels that act after iterations 1, 2, 4, 8.
+int enqueue_iteration(ac_batch *b, cudaStream_t s, unsigned long long cond, int use_cond, bool timed, bool rebase) {
     int rc;
+    const bool pdl = b->pdl;
     if (timed) CK(cudaEventRecord(b->ev[0], s));
     for (int st = 1; st <= b->opt.rk_stages; ++st) {
-        if ((rc = stage_launch(b, s, st, b->variant)) != AC_OK) return rc;
+        b->pdl = pdl && st > 1;   // the first stage waits for the iteration before to drain (see ac_api.cu)
+        rc = stage_launch(b, s, st, b->variant);
+        b->pdl = pdl;
+        if (rc != AC_OK) return rc;
         if (timed) CK(cudaEventRecord(b->ev[st], s));
     }
     CK(launch_pdl(b->pdl, batch_end_kernel<256>, dim3(b->n), dim3(256), 0, s, b->tanks_dev, b->sync, b->n, cond,
                   use_cond));
     CK(cudaGetLastError());
-    if (b->plevel) {
+    if (b->plevel && rebase) {
         CK(launch_pdl(b->pdl, batch_rebase_shift_kernel, b->rebase_grid, dim3(256), 0, s, b->tanks_dev));
         CK(launch_pdl(b->pdl, batch_rebase_jumps_kernel, b->rebase_grid, dim3(256), 0, s, b->tanks_dev));
     }
     return AC_OK;
 }
 
+// As the single tank's graph: with a pressure rebase the first kRebaseLast
+// iterations run in line ahead of the loop, the rebase kernels only where
+// they act (every tank still iterating is at the same iteration), and the
+// loop's body holds kLoopIters iterations without them.
 int build_graph(ac_batch *b) {
     if (b->exec) return AC_OK;
     CK(cudaGraphCreate(&b->graph, 0));
     cudaGraphConditionalHandle h;
     CK(cudaGraphConditionalHandleCreate(&h, b->graph, 1, cudaGraphCondAssignDefault));
+    std::vector<cudaGraphNode_t> pro;
+    int rc = AC_OK;
+    if (b->plevel) {
+        CK(cudaStreamBeginCaptureToGraph(b->cap, b->graph, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
+        for (int m = 1; m <= kRebaseLast && rc == AC_OK; ++m)
+            rc = enqueue_iteration(b, b->cap, (unsigned long long)h, 1, false, rebase_after(m));
+        cudaStreamCaptureStatus st;
+        cudaGraph_t g = nullptr, captured = nullptr;
+        const cudaGraphNode_t *deps = nullptr;
+        size_t nd = 0;
+        cudaError_t e = cudaStreamGetCaptureInfo(b->cap, &st, nullptr, &g, &deps, nullptr, &nd);
+        if (e == cudaSuccess) pro.assign(deps, deps + nd);
+        const cudaError_t e2 = cudaStreamEndCapture(b->cap, &captured);
+        if (rc != AC_OK) return rc;
+        if (e != cudaSuccess || e2 != cudaSuccess)
+            return fail(AC_ERR_CUDA, "graph capture failed: %s", cudaGetErrorString(e != cudaSuccess ? e : e2));
+    }
     alignas(cudaGraphNodeParams) unsigned char cp_raw[sizeof(cudaGraphNodeParams)];
     memset(cp_raw, 0, sizeof cp_raw);
     cudaGraphNodeParams &cp = *reinterpret_cast<cudaGraphNodeParams *>(cp_raw);
@@ -534,10 +559,11 @@ int build_graph(ac_batch *b) {
     cp.conditional.type = cudaGraphCondTypeWhile;
     cp.conditional.size = 1;
     cudaGraphNode_t node;
-    CK(cudaGraphAddNode(&node, b->graph, nullptr, nullptr, 0, &cp));
+    CK(cudaGraphAddNode(&node, b->graph, pro.empty() ? nullptr : pro.data(), nullptr, pro.size(), &cp));
     cudaGraph_t body = cp.conditional.phGraph_out[0];
     CK(cudaStreamBeginCaptureToGraph(b->cap, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-    const int rc = enqueue_iteration(b, b->cap, (unsigned long long)h, 1, false);
+    for (int m = 0; m < kLoopIters && rc == AC_OK; ++m)
+        rc = enqueue_iteration(b, b->cap, (unsigned long long)h, 1, false, false);
     cudaGraph_t captured = nullptr;
     const cudaError_t e = cudaStreamEndCapture(b->cap, &captured);
     if (rc != AC_OK) return rc;
@@ -859,7 +885,7 @@ static int batch_step_impl(ac_batch *b, const double *dt, double tol, int max_it
     long long iters_run = 0;
     if (b->profiling) {
         while (true) {
-            if ((rc = enqueue_iteration(b, s, 0, 0, true)) != AC_OK) return rc;
+            if ((rc = enqueue_iteration(b, s, 0, 0, true, true)) != AC_OK) return rc;
             CK(cudaMemcpyAsync(b->hctl, b->ctl, b->n * sizeof(Ctl), cudaMemcpyDeviceToHost, s));
             CK(cudaStreamSynchronize(s));
             for (int st = 1; st <= b->opt.rk_stages; ++st) {
@@ -880,7 +906,11 @@ static int batch_step_impl(ac_batch *b, const double *dt, double tol, int max_it
         CK(cudaStreamSynchronize(s));
         for (int k = 0; k < b->n; ++k) iters_run = std::max<long long>(iters_run, b->hctl[k].iter);
     }
-    b->launches += iters_run * (b->opt.rk_stages + 1 + (b->plevel ? 2 : 0));
+    if (b->profiling)
+        b->launches += iters_run * (b->opt.rk_stages + 1 + (b->plevel ? 2 : 0));
+    else   // the in-line iterations with their four rebase pairs, then whole bodies of the loop
+        b->launches += launched_iters(iters_run, b->plevel ? kRebaseLast : 0) * (b->opt.rk_stages + 1) +
+                       (b->plevel ? 8 : 0);
     int ret = AC_OK;
     bool any_nonfinite = false;
     for (int k = 0; k < b->n; ++k) {

@@ -22,7 +22,7 @@
 namespace acgb {
 
 // Device-resident control block of one physical step.
-struct Ctl {
+struct alignas(16) Ctl {
     int iter;        // pseudo-iterations completed
     int done;        // 1: stop iterating
     int cur;         // buffer index (0..2) holding Q^{m}
@@ -37,6 +37,25 @@ struct Ctl {
     int rebase;      // mixed form: fold the pressure increment into its FP64 level before the next iteration
     double tau, tau_end;  // pure pseudo-time run: pseudo-time reached and its end (+inf in a physical step)
 };
+
+// What every stage kernel needs of the control block, in two loads issued
+// together (the pass through L2 that each costs in sequence was 10 % of a small
+// grid's stage).
+template <typename T>
+struct CtlHead {
+    int done, cur;
+    T inv_dt;
+};
+template <typename T>
+__device__ __forceinline__ CtlHead<T> ctl_head(const Ctl *ctl) {
+    CtlHead<T> h;
+    int it, st;
+    double inv_dt;
+    asm volatile("ld.global.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(it), "=r"(h.done), "=r"(h.cur), "=r"(st) : "l"(ctl));
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(inv_dt) : "l"(&ctl->inv_dt));
+    h.inv_dt = T(inv_dt);
+    return h;
+}
 
 // The global pseudo-time step of the current iteration, shortened so that a
 // pure pseudo-time run lands on its end (tau_end is +inf otherwise).
@@ -134,13 +153,27 @@ __host__ __device__ __forceinline__ int final_buffer(int cur, int s_max) {
     return (s_max & 1) ? (cur + 1) % 3 : (cur + 2) % 3;
 }
 
+// Sum over a warp of four values per lane: lanes 0, 8, 16, 24 receive the sums
+// of v[0], v[1], v[2], v[3].  The first two exchanges leave each lane one of the
+// four, so that a warp spends 6 FP64 additions instead of 20.
+__device__ __forceinline__ double warp_sum4(const double v[4]) {
+    const int lane = threadIdx.x & 31;
+    const bool up16 = lane & 16, up8 = lane & 8;
+    double a = (up16 ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, up16 ? v[0] : v[2], 16);
+    const double b = (up16 ? v[3] : v[1]) + __shfl_xor_sync(0xffffffffu, up16 ? v[1] : v[3], 16);
+    a = (up8 ? b : a) + __shfl_xor_sync(0xffffffffu, up8 ? a : b, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    return a;
+}
+
 // Sum of the stage-1 residual partials (4 per slot, nparts slots) in a fixed
 // order: 128 strided sums, a shuffle tree in each of four warps, the four
 // warp sums left to right.  Called by every thread of a CTA of at least
-// kEndLanes threads; the sums are valid in thread 0.  The single-tank end of
-// iteration and the batch's per-tank end both use it, so a tank's norms do
+// kEndLanes threads; thread f < 4 receives field f's sum.  The single-tank end
+// of iteration and the batch's per-tank end both use it, so a tank's norms do
 // not depend on which of them ran.
-__device__ __forceinline__ void sum_partials_fixed(const double *partials, int nparts, double out[4]) {
+__device__ __forceinline__ double sum_partials_fixed(const double *partials, int nparts) {
     __shared__ double wsum[kEndLanes / 32][4];
     const int tid = threadIdx.x;
     if (tid < kEndLanes) {
@@ -149,63 +182,83 @@ __device__ __forceinline__ void sum_partials_fixed(const double *partials, int n
 #pragma unroll
             for (int f = 0; f < 4; ++f) s[f] += partials[(size_t)b * 4 + f];
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-            for (int f = 0; f < 4; ++f) s[f] += __shfl_down_sync(0xffffffffu, s[f], o);
-        }
-        if ((tid & 31) == 0) {
-#pragma unroll
-            for (int f = 0; f < 4; ++f) wsum[tid >> 5][f] = s[f];
-        }
+        const double v = warp_sum4(s);
+        if ((tid & 7) == 0) wsum[tid >> 5][(tid & 31) >> 3] = v;
     }
     __syncthreads();
-    if (tid == 0) {
-        for (int f = 0; f < 4; ++f) {
-            double sum = wsum[0][f];
-            for (int w = 1; w < kEndLanes / 32; ++w) sum += wsum[w][f];
-            out[f] = sum;
-        }
+    double sum = 0.0;
+    if (tid < 4) {
+        sum = wsum[0][tid];
+        for (int w = 1; w < kEndLanes / 32; ++w) sum += wsum[w][tid];
     }
+    return sum;
 }
+
+// The control block's part in the stopping test, read by threads f < 4 before
+// the partial sums (whose loads it overlaps) and judged by them after.
+struct EndTest {
+    int it, cur, max_iters, fixed;
+    double tol, R0, abs_tol;
+    bool finite, conv;
+    __device__ __forceinline__ void load(const Ctl *ctl) {
+        const int f = threadIdx.x;
+        if (f >= 4) return;
+        it = ctl->iter + 1;
+        cur = ctl->cur;
+        max_iters = ctl->max_iters;
+        fixed = ctl->fixed;
+        tol = ctl->tol;
+        R0 = ctl->R0[f];
+        abs_tol = ctl->abs_tol[f];
+    }
+    // threads f < 4 only: field f's norm, stored, and the test over all fields
+    __device__ __forceinline__ void judge(Ctl *ctl, double sum, double inv_cells) {
+        const int f = threadIdx.x;
+        const double R = sqrt(sum * inv_cells);
+        ctl->R[f] = R;
+        if (it == 1) ctl->R0[f] = R0 = R;
+        finite = __all_sync(0xfu, isfinite(R));
+        conv = __all_sync(0xfu, R <= fmax(tol * R0, abs_tol));
+    }
+};
 
 // End of a pseudo-iteration: the residual norms from the stage-1 partials,
 // the stopping test (Alg. 1), the buffer rotation and, inside a captured
 // loop, the while-condition.  Called by every thread of one CTA of at least
 // kEndLanes threads.
 __device__ __forceinline__ void end_iteration(Ctl *ctl, const double *partials, const IterEnd &e) {
-    double sums[4];
-    sum_partials_fixed(partials, e.nparts, sums);
+    EndTest t;
+    t.load(ctl);
+    double tau = 0.0, tau_end = 0.0, dtau = 0.0;
     const int tid = threadIdx.x;
     if (tid == 0) {
-        const int it = ctl->iter + 1;
-        ctl->iter = it;
-        bool finite = true, conv = true;
-        for (int f = 0; f < 4; ++f) {
-            const double R = sqrt(sums[f] * e.inv_cells);
-            ctl->R[f] = R;
-            if (it == 1) ctl->R0[f] = R;
-            if (!isfinite(R)) finite = false;
-            const double thr = fmax(ctl->tol * ctl->R0[f], ctl->abs_tol[f]);
-            if (!(R <= thr)) conv = false;
-        }
-        ctl->cur = final_buffer(ctl->cur, e.s_max);
+        tau = ctl->tau;
+        tau_end = ctl->tau_end;
+        dtau = global_dtau(ctl);
+    }
+    const double sum = sum_partials_fixed(partials, e.nparts);
+    if (tid >= 4) return;
+    t.judge(ctl, sum, e.inv_cells);
+    if (tid == 0) {
+        ctl->iter = t.it;
+        ctl->cur = final_buffer(t.cur, e.s_max);
         bool reached = false;   // a pure pseudo-time run reached its end
-        if (ctl->tau_end < INFINITY) {
-            ctl->tau += global_dtau(ctl);
-            reached = ctl->tau >= ctl->tau_end;
+        if (tau_end < INFINITY) {
+            tau += dtau;
+            ctl->tau = tau;
+            reached = tau >= tau_end;
         }
         int done = 0;
-        if (!finite) { ctl->status = -3; done = 1; }
+        if (!t.finite) { ctl->status = -3; done = 1; }
         else if (reached) { ctl->status = 0; done = 1; }
-        else if (!ctl->fixed && conv) { ctl->status = 0; done = 1; }
-        else if (it >= ctl->max_iters) {
+        else if (!t.fixed && t.conv) { ctl->status = 0; done = 1; }
+        else if (t.it >= t.max_iters) {
             // a fixed iteration count is complete; a pseudo-time run short of its end is not
-            ctl->status = (ctl->fixed && !(ctl->tau_end < INFINITY)) ? 0 : 1;
+            ctl->status = (t.fixed && !(tau_end < INFINITY)) ? 0 : 1;
             done = 1;
         }
         ctl->done = done;
-        ctl->rebase = (e.rebase_pow2 && !done && rebase_after(it)) ? 1 : 0;
+        ctl->rebase = (e.rebase_pow2 && !done && rebase_after(t.it)) ? 1 : 0;
         ctl->dtau_bits = 0x7ff0000000000000ull;
         if (e.use_cond) cudaGraphSetConditional(e.cond, done ? 0u : 1u);
     }
@@ -277,14 +330,15 @@ stage_kernel(const SweepArgs<T> a) {
     pdl_trigger();
     pdl_wait();
     const Ctl *ctl = a.ctl;
-    if (ctl->done) return;
+    const CtlHead<T> head = ctl_head<T>(ctl);
+    if (head.done) return;
     int in, out;
-    const int cur = ctl->cur;
+    const int cur = head.cur;
     stage_buffers(cur, a.stage, in, out);
     const T *const *qin = a.buf[in];
     const T *const *q0 = a.buf[cur];
     T *const *qout = a.buf[out];
-    const T inv_dt = a.realtime ? T(ctl->inv_dt) : T(0);
+    const T inv_dt = a.realtime ? head.inv_dt : T(0);
 
     const int nx = a.nx, ny = a.ny;
     const int tid = threadIdx.x;
@@ -618,17 +672,9 @@ stage_kernel(const SweepArgs<T> a) {
         }
     }
     if (a.stage == 1) {
-        // deterministic block reduction of the squared bracket (FP64): the
-        // first two exchanges leave each lane one of the four sums, so a warp
-        // spends 6 additions instead of 20
-        const int lane = tid & 31;
-        const bool up16 = lane & 16, up8 = lane & 8;
-        double v0 = (up16 ? sq[2] : sq[0]) + __shfl_xor_sync(0xffffffffu, up16 ? sq[0] : sq[2], 16);
-        const double v1 = (up16 ? sq[3] : sq[1]) + __shfl_xor_sync(0xffffffffu, up16 ? sq[1] : sq[3], 16);
-        v0 = (up8 ? v1 : v0) + __shfl_xor_sync(0xffffffffu, up8 ? v0 : v1, 8);
-#pragma unroll
-        for (int o = 4; o > 0; o >>= 1) v0 += __shfl_xor_sync(0xffffffffu, v0, o);
-        if ((lane & 7) == 0) sm.red[lane >> 3][tid >> 5] = v0;   // field 2 (lane/16) + (lane/8 mod 2)
+        // deterministic block reduction of the squared bracket (FP64)
+        const double v = warp_sum4(sq);
+        if ((tid & 7) == 0) sm.red[(tid & 31) >> 3][tid >> 5] = v;
         __syncthreads();
         if (tid < 4) {
             double s = 0.0;

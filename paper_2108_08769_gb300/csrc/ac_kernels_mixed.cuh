@@ -153,7 +153,9 @@ struct CellLoad {
     const float4 *__restrict__ qn;
     const float4 *__restrict__ d;
     __device__ __forceinline__ float4 operator()(int s, bool fx, bool fy) const {
-        const float4 q = __ldg(qn + s), e = d[s];
+        return form(__ldg(qn + s), d[s], fx, fy);
+    }
+    static __device__ __forceinline__ float4 form(const float4 &q, const float4 &e, bool fx, bool fy) {
         const float r = q.x + e.x;
         float m = q.y + e.y;
         float n = q.z + e.z;
@@ -438,16 +440,16 @@ struct PrefetchSrc {
 // RAW_AUX: the ring holds (dQ of rho u, dQ of rho v, rho_ref, fold bits) as
 // copied, and the real-time terms are formed here (Backward-Euler only).
 template <int TX, int TY, int NT, int RS, bool BDF, bool RAW_AUX, typename Src>
-__device__ __forceinline__ void mixed_tile_compute(const MixedArgs &a, int stage, float alpha, int x0, int y0,
-                                                   bool interior, double *partial, MixedSmem<TX, TY> &sm, Src &src) {
+__device__ __forceinline__ void mixed_tile_compute(const MixedArgs &a, const CtlHead<float> &head, int stage, float alpha,
+                                                   int x0, int y0, bool interior, double *partial,
+                                                   MixedSmem<TX, TY> &sm, Src &src) {
     static_assert(!(RAW_AUX && BDF), "raw ring terms are Backward-Euler only");
     using S = MixedSmem<TX, TY>;
     constexpr int RW = S::RW, GW = S::GW, GH = S::GH;
-    const Ctl *ctl = a.ctl;
     int in, out;
-    stage_buffers(ctl->cur, stage, in, out);
+    stage_buffers(head.cur, stage, in, out);
     float4 *dout = a.d[out];
-    const float inv_dt = a.realtime ? float(ctl->inv_dt) : 0.0f;
+    const float inv_dt = a.realtime ? head.inv_dt : 0.0f;
     const int nx = a.nx, ny = a.ny;
     const int tid = threadIdx.x;
     const bool new_gradp = (a.gradp == kGradNew);
@@ -580,21 +582,20 @@ __device__ __forceinline__ void mixed_tile_compute(const MixedArgs &a, int stage
 // reference jumps are copied with cp.async while the halo is being loaded,
 // and the update's own-cell inputs are prefetched at the start of phase 3.
 template <int TX, int TY, int NT, int RS, bool BDF, bool PF = false>
-__device__ __forceinline__ void mixed_tile(const MixedArgs &a, int stage, float alpha, int bx, int by,
-                                           double *partial, unsigned char *smem_raw) {
+__device__ __forceinline__ void mixed_tile(const MixedArgs &a, const CtlHead<float> &head, int stage, float alpha, int bx,
+                                           int by, double *partial, unsigned char *smem_raw) {
     using S = MixedSmem<TX, TY>;
     static_assert((TX * TY) % NT == 0 && NT % 32 == 0, "tile/thread shape");
     static_assert(!PF || (NT == TX * TY && !BDF), "prefetch: one cell per thread, Backward-Euler");
     S &sm = *reinterpret_cast<S *>(smem_raw);
     constexpr int RW = S::RW, RH = S::RH, GW = S::GW, GH = S::GH;
 
-    const Ctl *ctl = a.ctl;
     int in, out;
-    const int cur = ctl->cur;
+    const int cur = head.cur;
     stage_buffers(cur, stage, in, out);
     const float4 *din = a.d[in];
     const float4 *d0 = a.d[cur];
-    const float inv_dt = a.realtime ? float(ctl->inv_dt) : 0.0f;
+    const float inv_dt = a.realtime ? head.inv_dt : 0.0f;
 
     const int nx = a.nx, ny = a.ny;
     const int tid = threadIdx.x;
@@ -605,6 +606,21 @@ __device__ __forceinline__ void mixed_tile(const MixedArgs &a, int stage, float 
     const bool new_gradp = (a.gradp == kGradNew);
     const bool need_rt = new_gradp && a.realtime;
 
+    // Interior tiles of the prefetching form start their halo's loads first, so
+    // that the index arithmetic of the copies below runs under their latency.
+    constexpr int NW = (RW * RH + NT - 1) / NT;
+    float4 wq[NW], wd[NW];
+    if (PF && interior) {
+        const int base = (y0 - 2) * nx + (x0 - 2);
+#pragma unroll
+        for (int r = 0; r < NW; ++r) {
+            const int k = tid + r * NT;
+            if (k >= RW * RH) continue;
+            const int s = base + (k / RW) * nx + k % RW;
+            wq[r] = __ldg(a.qn + s);
+            wd[r] = din[s];
+        }
+    }
     if constexpr (PF) {
         // face level jumps (zero outside the domain, as x_face_jump, y_face_jump)
         const bool per_x = (a.bc[0] == kPeriodic), per_y = (a.bc[2] == kPeriodic);
@@ -648,7 +664,11 @@ __device__ __forceinline__ void mixed_tile(const MixedArgs &a, int stage, float 
     }
 
     // ---- 1. stage Q^{s-1} = Q^n + dQ^{s-1} (+ halo) as W = (rho, u, v, dp) ----
-    if (interior) {
+    if (PF && interior) {
+#pragma unroll
+        for (int r = 0; r < NW; ++r)
+            if (tid + r * NT < RW * RH) sm.w[tid + r * NT] = CellLoad::form(wq[r], wd[r], false, false);
+    } else if (interior) {
         const int base = (y0 - 2) * nx + (x0 - 2);
         for (int k = tid; k < RW * RH; k += NT) {
             const int rr = k / RW, cc = k - rr * RW;
@@ -703,11 +723,11 @@ __device__ __forceinline__ void mixed_tile(const MixedArgs &a, int stage, float 
         cp_async_wait_all();
         __syncthreads();
         PrefetchSrc src{a, d0, {}};
-        mixed_tile_compute<TX, TY, NT, RS, BDF, true>(a, stage, alpha, x0, y0, interior, partial, sm, src);
+        mixed_tile_compute<TX, TY, NT, RS, BDF, true>(a, head, stage, alpha, x0, y0, interior, partial, sm, src);
     } else {
         __syncthreads();
         DirectSrc src{a, d0};
-        mixed_tile_compute<TX, TY, NT, RS, BDF, false>(a, stage, alpha, x0, y0, interior, partial, sm, src);
+        mixed_tile_compute<TX, TY, NT, RS, BDF, false>(a, head, stage, alpha, x0, y0, interior, partial, sm, src);
     }
 }
 
@@ -717,8 +737,9 @@ stage_kernel_mixed(const MixedArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     pdl_trigger();
     pdl_wait();
-    if (a.ctl->done) return;
-    mixed_tile<TX, TY, NT, RS, BDF, PF>(a, a.stage, a.alpha, blockIdx.x, blockIdx.y,
+    const CtlHead<float> head = ctl_head<float>(a.ctl);
+    if (head.done) return;
+    mixed_tile<TX, TY, NT, RS, BDF, PF>(a, head, a.stage, a.alpha, blockIdx.x, blockIdx.y,
                            a.partials + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * 4, smem_raw);
 }
 
@@ -805,23 +826,22 @@ struct HeldSrc {
 // windows reach ghost rows; the main loop then tests neither the row number
 // nor the fold of ghost rows.
 template <int H, int UNROLL = 1, int SK = 0>
-__device__ __forceinline__ void mixed_strip(const MixedArgs &a, int stage, float alpha, int sx, int sy,
-                                            double *partial, StripRing *ring) {
+__device__ __forceinline__ void mixed_strip(const MixedArgs &a, const CtlHead<float> &head, int stage, float alpha, int sx,
+                                            int sy, double *partial, StripRing *ring) {
     constexpr bool FAST = SK != 0;
     const bool st1 = SK == 0 ? (stage == 1) : (SK == 1);
-    const Ctl *ctl = a.ctl;
     const int lane = threadIdx.x & 31;
     const int nx = a.nx, ny = a.ny;
     const int c = sx * kStripOut + lane - 2;   // this lane's column
     const int y0 = sy * H, y1 = min(y0 + H, ny);
     int in, out;
-    const int cur = ctl->cur;
+    const int cur = head.cur;
     stage_buffers(cur, stage, in, out);
     const float4 *din = a.d[in];
     const float4 *d0 = a.d[cur];
     float4 *dout = a.d[out];
     const bool need_rt = FAST || a.realtime != 0;
-    const float inv_dt = need_rt ? float(ctl->inv_dt) : 0.0f;
+    const float inv_dt = need_rt ? head.inv_dt : 0.0f;
     const float b0dt = a.B0 * inv_dt;
     const int klim = FAST ? 1 : a.limiter_k;
     const bool per_x = (a.bc[0] == kPeriodic);
@@ -1023,12 +1043,13 @@ __global__ void __launch_bounds__(WPC * 32, MINB)
 sweep_kernel_mixed(const MixedArgs a, int strips_x, int nstrips) {
     pdl_trigger();
     pdl_wait();
-    if (a.ctl->done) return;
+    const CtlHead<float> head = ctl_head<float>(a.ctl);
+    if (head.done) return;
     extern __shared__ __align__(16) unsigned char strip_smem[];
     const int warp = blockIdx.x * WPC + (threadIdx.x >> 5);
     if (warp >= nstrips) return;   // whole warps only
     const int sy = warp / strips_x, sx = warp - sy * strips_x;
-    mixed_strip<H, SK == 1 ? 1 : 2, SK>(a, a.stage, a.alpha, sx, sy, a.partials + (size_t)warp * 4,
+    mixed_strip<H, SK == 1 ? 1 : 2, SK>(a, head, a.stage, a.alpha, sx, sy, a.partials + (size_t)warp * 4,
                       reinterpret_cast<StripRing *>(strip_smem) + (threadIdx.x >> 5));
 }
 
