@@ -594,7 +594,7 @@ struct MixedBackend : Backend {
         a.riemann = c->opt.riemann;
         a.local_dtau = c->opt.local_dtau; a.alpha_pi_p_row = c->opt.alpha_pi_p_row;
         a.stage = stage; a.s_max = c->opt.rk_stages;
-        a.alpha = stage > 0 ? float(1.0 / double(c->opt.rk_stages - stage + 1)) : 0.0f;
+        a.inv_alpha = float(c->opt.rk_stages - stage + 1);
         const double dx = c->dx, dy = c->dy;
         a.dx = float(dx); a.dy = float(dy); a.half_dx = float(0.5 * dx); a.half_dy = float(0.5 * dy);
         a.inv_dx = float(1.0 / dx); a.inv_dy = float(1.0 / dy);
@@ -603,6 +603,7 @@ struct MixedBackend : Backend {
         a.beta = float(c->beta); a.inv_beta = float(1.0 / c->beta);
         a.gx = float(c->grid.gx); a.gy = float(c->grid.gy);
         a.cfl_area = float(c->opt.cfl_tau * dx * dy);
+        a.inv_cfl_area = float(1.0 / (c->opt.cfl_tau * dx * dy));
         a.plevel = plevel ? 1 : 0;
         for (int b = 0; b < 3; ++b) a.d[b] = d[b];
         a.qn = qn;

@@ -69,7 +69,7 @@ __constant__ BatchTank c_tanks[kConstTanks];
 // ac_api.cu.)
 template <int TX, int TY, int NT, int RS = kOsher, bool BDF = false, bool CD = false, bool PF = false>
 __global__ void __launch_bounds__(NT, NT == 512 ? 3 : 6)
-batch_stage_kernel(const BatchTank *__restrict__ tanks, const int *__restrict__ tile_tank, int stage, float alpha,
+batch_stage_kernel(const BatchTank *__restrict__ tanks, const int *__restrict__ tile_tank, int stage, float inv_alpha,
                    int slot0) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     pdl_trigger();
@@ -81,14 +81,14 @@ batch_stage_kernel(const BatchTank *__restrict__ tanks, const int *__restrict__ 
         if (head.done) return;
         const int local = blockIdx.x - t.tile0;
         const int by = local / t.tiles_x, bx = local - by * t.tiles_x;
-        mixed_tile<TX, TY, NT, RS, BDF, PF>(t.a, head, stage, alpha, bx, by, t.a.partials + (size_t)local * 4, smem_raw);
+        mixed_tile<TX, TY, NT, RS, BDF, PF>(t.a, head, stage, inv_alpha, bx, by, t.a.partials + (size_t)local * 4, smem_raw);
     } else {
         const BatchTank &t = tanks[k];
         const CtlHead<float> head = ctl_head<float>(t.a.ctl);
         if (head.done) return;
         const int local = blockIdx.x - t.tile0;
         const int by = local / t.tiles_x, bx = local - by * t.tiles_x;
-        mixed_tile<TX, TY, NT, RS, BDF, PF>(t.a, head, stage, alpha, bx, by, t.a.partials + (size_t)local * 4, smem_raw);
+        mixed_tile<TX, TY, NT, RS, BDF, PF>(t.a, head, stage, inv_alpha, bx, by, t.a.partials + (size_t)local * 4, smem_raw);
     }
 }
 
@@ -98,7 +98,7 @@ batch_stage_kernel(const BatchTank *__restrict__ tanks, const int *__restrict__ 
 template <int H, int WPC, int MINB, bool CD, int SK>
 __global__ void __launch_bounds__(WPC * 32, MINB)
 batch_sweep_kernel(const BatchTank *__restrict__ tanks, const int *__restrict__ strip_tank, int nstrips, int stage,
-                   float alpha, int slot0) {
+                   float inv_alpha, int slot0) {
     extern __shared__ __align__(16) unsigned char strip_smem[];
     StripRing *ring = reinterpret_cast<StripRing *>(strip_smem) + (threadIdx.x >> 5);
     pdl_trigger();
@@ -112,14 +112,14 @@ batch_sweep_kernel(const BatchTank *__restrict__ tanks, const int *__restrict__ 
         if (head.done) return;
         const int local = w - t.tile0;
         const int sy = local / t.tiles_x, sx = local - sy * t.tiles_x;
-        mixed_strip<H, 1, SK>(t.a, head, stage, alpha, sx, sy, t.a.partials + (size_t)local * 4, ring);
+        mixed_strip<H, 1, SK>(t.a, head, stage, inv_alpha, sx, sy, t.a.partials + (size_t)local * 4, ring);
     } else {
         const BatchTank &t = tanks[k];
         const CtlHead<float> head = ctl_head<float>(t.a.ctl);
         if (head.done) return;
         const int local = w - t.tile0;
         const int sy = local / t.tiles_x, sx = local - sy * t.tiles_x;
-        mixed_strip<H, 1, SK>(t.a, head, stage, alpha, sx, sy, t.a.partials + (size_t)local * 4, ring);
+        mixed_strip<H, 1, SK>(t.a, head, stage, inv_alpha, sx, sy, t.a.partials + (size_t)local * 4, ring);
     }
 }
 
@@ -269,34 +269,34 @@ cudaError_t allow_smem() {
 
 // slot0 < 0: descriptors in global memory
 template <int H, int WPC, int MINB, int SK>
-cudaError_t launch_sweep_sk(const BatchTank *tanks, const int *map, int nstrips, int stage, float alpha, int slot0,
+cudaError_t launch_sweep_sk(const BatchTank *tanks, const int *map, int nstrips, int stage, float inv_alpha, int slot0,
                             bool pdl, cudaStream_t s) {
     const dim3 g((nstrips + WPC - 1) / WPC);
     const size_t smem = WPC * sizeof(StripRing);
     const dim3 b(WPC * 32);
     if (slot0 >= 0)
         return launch_pdl(pdl, batch_sweep_kernel<H, WPC, MINB, true, SK>, g, b, smem, s, tanks, map, nstrips, stage,
-                          alpha, slot0);
+                          inv_alpha, slot0);
     return launch_pdl(pdl, batch_sweep_kernel<H, WPC, MINB, false, SK>, g, b, smem, s, tanks, map, nstrips, stage,
-                      alpha, 0);
+                      inv_alpha, 0);
 }
 // fast: the batch runs the default options (see mixed_strip)
 template <int H, int WPC, int MINB>
-cudaError_t launch_sweep(const BatchTank *tanks, const int *map, int nstrips, int stage, float alpha, int slot0,
+cudaError_t launch_sweep(const BatchTank *tanks, const int *map, int nstrips, int stage, float inv_alpha, int slot0,
                          bool fast, bool pdl, cudaStream_t s) {
-    if (!fast) return launch_sweep_sk<H, WPC, MINB, 0>(tanks, map, nstrips, stage, alpha, slot0, pdl, s);
-    if (stage == 1) return launch_sweep_sk<H, WPC, MINB, 1>(tanks, map, nstrips, stage, alpha, slot0, pdl, s);
-    return launch_sweep_sk<H, WPC, MINB, 2>(tanks, map, nstrips, stage, alpha, slot0, pdl, s);
+    if (!fast) return launch_sweep_sk<H, WPC, MINB, 0>(tanks, map, nstrips, stage, inv_alpha, slot0, pdl, s);
+    if (stage == 1) return launch_sweep_sk<H, WPC, MINB, 1>(tanks, map, nstrips, stage, inv_alpha, slot0, pdl, s);
+    return launch_sweep_sk<H, WPC, MINB, 2>(tanks, map, nstrips, stage, inv_alpha, slot0, pdl, s);
 }
 
 template <int TX, int TY, int NT, int RS = kOsher, bool BDF = false, bool PF = false>
-cudaError_t launch_stage(const BatchTank *tanks, const int *map, int ntiles, int stage, float alpha, int slot0,
+cudaError_t launch_stage(const BatchTank *tanks, const int *map, int ntiles, int stage, float inv_alpha, int slot0,
                          bool pdl, cudaStream_t s) {
     if (slot0 >= 0)
         return launch_pdl(pdl, batch_stage_kernel<TX, TY, NT, RS, BDF, true, PF>, dim3(ntiles), dim3(NT),
-                          sizeof(MixedSmem<TX, TY>), s, tanks, map, stage, alpha, slot0);
+                          sizeof(MixedSmem<TX, TY>), s, tanks, map, stage, inv_alpha, slot0);
     return launch_pdl(pdl, batch_stage_kernel<TX, TY, NT, RS, BDF, false, PF>, dim3(ntiles), dim3(NT),
-                      sizeof(MixedSmem<TX, TY>), s, tanks, map, stage, alpha, 0);
+                      sizeof(MixedSmem<TX, TY>), s, tanks, map, stage, inv_alpha, 0);
 }
 
 // First-fit allocator over the constant descriptor table (process-wide).
@@ -413,25 +413,25 @@ struct StageLaunch {
     const BatchTank *tanks;
     const int *map;
     int ntiles, stage;
-    float alpha;
+    float inv_alpha;
     int slot0;
     bool fast, pdl;
     template <int TX, int TY, int NT, int RS = kOsher, bool BDF = false, bool PF = false>
     cudaError_t go(cudaStream_t s) const {
-        return launch_stage<TX, TY, NT, RS, BDF, PF>(tanks, map, ntiles, stage, alpha, slot0, pdl, s);
+        return launch_stage<TX, TY, NT, RS, BDF, PF>(tanks, map, ntiles, stage, inv_alpha, slot0, pdl, s);
     }
     template <int H, int MINB = 4>
     cudaError_t strips(cudaStream_t s) const {
-        return launch_sweep<H, 4, MINB>(tanks, map, ntiles, stage, alpha, slot0, fast, pdl, s);
+        return launch_sweep<H, 4, MINB>(tanks, map, ntiles, stage, inv_alpha, slot0, fast, pdl, s);
     }
 };
 
 int stage_launch(ac_batch *b, cudaStream_t s, int stage, int v) {
     cudaError_t e;
-    const float alpha = float(1.0 / double(b->opt.rk_stages - stage + 1));   // alpha_s
+    const float inv_alpha = float(b->opt.rk_stages - stage + 1);   // 1/alpha_s
     // the batch's tanks all use the pseudo-time step of their own cells
     const bool fast = b->opt.limiter_k == 1 && b->opt.realtime && b->opt.alpha_pi_p_row;
-    const StageLaunch L{b->tanks_dev, b->tile_map, b->ntiles, stage, alpha, b->slot0, fast, b->pdl};
+    const StageLaunch L{b->tanks_dev, b->tile_map, b->ntiles, stage, inv_alpha, b->slot0, fast, b->pdl};
     // the Bassi and Roe fluxes are compiled for the first tile shape only
     if (b->opt.riemann == AC_RIEMANN_BASSI) e = L.go<32, 8, 256, kBassi, true>(s);
     else if (b->opt.riemann == AC_RIEMANN_ROE) e = L.go<32, 8, 256, kRoe, true>(s);
@@ -738,6 +738,7 @@ int ac_batch_create(int n, const ac_grid *grids, const double *beta, const ac_bc
         a.beta = float(beta[k]); a.inv_beta = float(1.0 / beta[k]);
         a.gx = float(g.gx); a.gy = float(g.gy);
         a.cfl_area = float(o.cfl_tau * dx * dy);
+        a.inv_cfl_area = float(1.0 / (o.cfl_tau * dx * dy));
         a.plevel = b->plevel ? 1 : 0;
         b->use_ref[k] = mixed_uses_reference(bcs[k], o.gradp);
         for (int x = 0; x < 3; ++x) a.d[x] = b->d[x] + pos;

@@ -53,17 +53,17 @@ struct MixedArgs {
     int gradp, limiter_k, realtime, local_dtau, alpha_pi_p_row;
     int riemann;           // kOsher / kBassi / kRoe
     int stage, s_max;
-    float alpha;
+    float inv_alpha;       // 1/alpha_s
     float dx, dy, half_dx, half_dy, inv_dx, inv_dy, dx_over_dy, dy_over_dx;
     float nh_inv_dx, nh_inv_dy;   // -1/(2 dx), -1/(2 dy)
     float beta, inv_beta, gx, gy;
-    float cfl_area;
+    float cfl_area, inv_cfl_area;
     int plevel;            // 1: pressure as dp over the FP64 level p^n; 0: the record holds p
     float4 *d[3];          // per cell (dQ of rho, rho u, rho v; dp or p), three rotating buffers
     float4 *qn;            // per cell (FP32 Q^n of rho, rho u, rho v; rho_ref)
     float2 *jmp;           // per cell (level jump across the west face, across the south face)
     float *lev_p;          // p at the start of the physical step (plevel = 0, for a restore)
-    float *dtau;           // per cell local pseudo-time step of the pseudo-iteration: written by stage 1 of
+    float *dtau;           // per cell inverse of the pseudo-iteration's local pseudo-time step: written by stage 1 of
                            // the column-strip sweep with the default options, read by its later stages
     float *D1[3], *D2[3];  // Q^n - Q^{n-1}, Q^n - Q^{n-2} (rho, rho u, rho v) for BDF2/BDF3
     int order;             // backward-difference order used in this step (1..3)
@@ -217,19 +217,30 @@ __device__ __forceinline__ void limit_diffs(float er, float wr, float nr, float 
 // column-strip sweep, so that both compute every value the same way.
 // ---------------------------------------------------------------------------
 
+// Eq. new_gradp times the spacings ex, ey, from slopes over the same
+// spacings: d(rho u u) = u A + rho u du with A = d(rho u) along x,
+// d(rho u v) = v A + rho u dv, and so on (20 operations instead of 27 term by
+// term).  The reference slope rho_ref g_y is removed from p's.
+__device__ __forceinline__ void gradp_slopes(const MixedArgs &a, const float4 &Wc, float srx, float sry, float sux,
+                                             float suy, float svx, float svy, float rtx, float rty, float rref,
+                                             float sg, float ex, float ey, float &spx, float &spy) {
+    const float rho = Wc.x, u = Wc.y, v = Wc.z, ru = rho * u, rv = rho * v;
+    const float A = fmaf(rho, sux, u * srx), B = fmaf(rho, svy, v * sry);
+    const float xx = fmaf(u, A, ru * sux), xy = fmaf(u, B, rv * suy);
+    const float yy = fmaf(v, B, rv * svy), yx = fmaf(v, A, ru * svx);
+    const float rd = rho - rref;
+    spx = fmaf(-a.dx_over_dy, xy, fmaf(ex, fmaf(sg < 0.0f ? -rho : rho, a.gx, -rtx), -xx));
+    spy = fmaf(-a.dy_over_dx, yx, fmaf(ey, fmaf(sg < 0.0f ? -rd : rd, a.gy, -rty), -yy));
+}
+
 // Half slope of p from the new pressure gradient (Eq. new_gradp) at a cell
 // with W = Wc, the half slopes of rho, u, v, the frozen real-time terms of
 // rho u, rho v (rtx, rty), the reference density and the ghost gravity sign.
 __device__ __forceinline__ void new_gradp_half_slopes(const MixedArgs &a, const float4 &Wc, float hrx, float hry,
                                                       float hux, float huy, float hvx, float hvy, float rtx,
                                                       float rty, float rref, float sg, float &hpx, float &hpy) {
-    const float rho = Wc.x, u = Wc.y, v = Wc.z;
-    const float ru = rho * u, rv = rho * v, uv = u * v;
-    hpx = -a.half_dx * rtx - (u * u * hrx + 2.0f * ru * hux) -
-          a.dx_over_dy * (uv * hry + ru * hvy + rv * huy) + a.half_dx * rho * a.gx * sg;
-    // slope of p - p_ref: the reference slope rho_ref g_y is removed
-    hpy = -a.half_dy * rty - (v * v * hry + 2.0f * rv * hvy) -
-          a.dy_over_dx * (uv * hrx + rv * hux + ru * hvx) + a.half_dy * (rho - rref) * a.gy * sg;
+    // half of the whole slopes, exactly: every term is a product with one half slope or half spacing
+    gradp_slopes(a, Wc, hrx, hry, hux, huy, hvx, hvy, rtx, rty, rref, sg, a.half_dx, a.half_dy, hpx, hpy);
 }
 
 // The same, whole slope of p - p_ref (twice the above, exactly: every term is
@@ -237,12 +248,7 @@ __device__ __forceinline__ void new_gradp_half_slopes(const MixedArgs &a, const 
 __device__ __forceinline__ void new_gradp_whole_slopes(const MixedArgs &a, const float4 &Wc, float srx, float sry,
                                                        float sux, float suy, float svx, float svy, float rtx,
                                                        float rty, float rref, float sg, float &spx, float &spy) {
-    const float rho = Wc.x, u = Wc.y, v = Wc.z;
-    const float ru = rho * u, rv = rho * v, uv = u * v;
-    spx = -a.dx * rtx - (u * u * srx + 2.0f * ru * sux) -
-          a.dx_over_dy * (uv * sry + ru * svy + rv * suy) + a.dx * rho * a.gx * sg;
-    spy = -a.dy * rty - (v * v * sry + 2.0f * rv * svy) -
-          a.dy_over_dx * (uv * srx + rv * sux + ru * svx) + a.dy * (rho - rref) * a.gy * sg;
+    gradp_slopes(a, Wc, srx, sry, sux, suy, svx, svy, rtx, rty, rref, sg, a.dx, a.dy, spx, spy);
 }
 
 // Face states between cells A (left/below) and B with half slopes SA, SB
@@ -295,11 +301,11 @@ __device__ __forceinline__ float4 face_flux(const MixedArgs &a, bool isx, const 
 // (a halo lane of the column-strip sweep, on a real cell's values) but
 // nothing is stored or summed.  FAST: the default options (local pseudo-time
 // step, alpha_PI on the p row) are compiled in rather than read.  DTM: 0
-// forms the local pseudo-time step from Q^{m}; 1 forms it and stores it in
-// a.dtau (stage 1); 2 takes it from dt_in, as stage 1 stored it (the later
-// stages: Q^{m} is the same for every stage of a pseudo-iteration).
+// forms the inverse of the local pseudo-time step from Q^{m}; 1 forms it and
+// stores it in a.dtau (stage 1); 2 takes it from dt_in, as stage 1 stored it
+// (the later stages: Q^{m} is the same for every stage of a pseudo-iteration).
 template <bool BDF, bool FAST = false, int DTM = 0, typename Src, typename Sq>
-__device__ __forceinline__ void cell_update(const MixedArgs &a, float alpha, float inv_dt, float b0dt, bool stage1,
+__device__ __forceinline__ void cell_update(const MixedArgs &a, float inv_alpha, float inv_dt, float b0dt, bool stage1,
                                             float4 *dout, int cell, int g, const float4 &Fw, const float4 &Fe,
                                             const float4 &Fs, const float4 &Fn, float fdx, float fdy, float jw,
                                             float je, float js, float jn, const Src &src, Sq &sq,
@@ -343,25 +349,24 @@ __device__ __forceinline__ void cell_update(const MixedArgs &a, float alpha, flo
     const float b1 = fmaf(je + jw, a.nh_inv_dx, fmaf(r0, a.gx, -div1 - rt1));
     const float b2 = fmaf(jn + js, a.nh_inv_dy, fmaf(r0 - rref, a.gy, -div2 - rt2));
     const float b3 = -div3;
-    float dtau;
+    // 1/dtau: Eq. point_implicit's alpha dtau / (1 + B0 alpha dtau/dt) is 1 / (1/(alpha dtau) + B0/dt)
+    float idt;
     if constexpr (DTM == 2) {
-        dtau = dt_in;
+        idt = dt_in;
     } else if (FAST || a.local_dtau) {
         const float ir = Ar<float>::rcp(r0);
         const float u = m0 * ir, v = n0 * ir, fb = 4.0f * a.beta * ir;
         const float u2 = u * u + fb, v2 = v * v + fb;
         const float cx = u2 * rsqrtf(u2), cy = v2 * rsqrtf(v2);
-        const float den = 0.5f * (fabsf(u) + cx) * a.dy + 0.5f * (fabsf(v) + cy) * a.dx;
-        dtau = __fdividef(a.cfl_area, den);
+        idt = fmaf(fabsf(u) + cx, a.half_dy, (fabsf(v) + cy) * a.half_dx) * a.inv_cfl_area;
         if constexpr (DTM == 1) {
-            if (live) a.dtau[g] = dtau;
+            if (live) a.dtau[g] = idt;
         }
     } else {
-        dtau = float(global_dtau(a.ctl));
+        idt = Ar<float>::rcp(float(global_dtau(a.ctl)));
     }
-    const float adt = alpha * dtau;
-    const float coef = __fdividef(adt, fmaf(adt, b0dt, 1.0f));   // Eq. point_implicit
-    const float coef_p = (FAST || a.alpha_pi_p_row) ? coef : adt;
+    const float coef = Ar<float>::rcp(fmaf(idt, inv_alpha, b0dt));
+    const float coef_p = (FAST || a.alpha_pi_p_row) ? coef : Ar<float>::rcp(idt * inv_alpha);
     if (live) dout[g] = make_float4(e0 + coef * b0, e1 + coef * b1, e2 + coef * b2, p0 + a.beta * coef_p * b3);
     if (stage1) {
         if (live) sq.add(b0, b1, b2, a.beta * b3);   // the p row in pressure units
@@ -440,7 +445,7 @@ struct PrefetchSrc {
 // RAW_AUX: the ring holds (dQ of rho u, dQ of rho v, rho_ref, fold bits) as
 // copied, and the real-time terms are formed here (Backward-Euler only).
 template <int TX, int TY, int NT, int RS, bool BDF, bool RAW_AUX, typename Src>
-__device__ __forceinline__ void mixed_tile_compute(const MixedArgs &a, const CtlHead<float> &head, int stage, float alpha,
+__device__ __forceinline__ void mixed_tile_compute(const MixedArgs &a, const CtlHead<float> &head, int stage, float inv_alpha,
                                                    int x0, int y0, bool interior, double *partial,
                                                    MixedSmem<TX, TY> &sm, Src &src) {
     static_assert(!(RAW_AUX && BDF), "raw ring terms are Backward-Euler only");
@@ -551,7 +556,7 @@ __device__ __forceinline__ void mixed_tile_compute(const MixedArgs &a, const Ctl
         if (gi >= nx || gj >= ny) continue;
         const int g = gj * nx + gi;
         const int fw = lj * (TX + 1) + li;
-        cell_update<BDF>(a, alpha, inv_dt, a.B0 * inv_dt, stage == 1, dout, cell, g, sm.fx[fw], sm.fx[fw + 1],
+        cell_update<BDF>(a, inv_alpha, inv_dt, a.B0 * inv_dt, stage == 1, dout, cell, g, sm.fx[fw], sm.fx[fw + 1],
                          sm.fy[cell], sm.fy[cell + TX], a.inv_dx, a.inv_dy, sm.dxf[fw], sm.dxf[fw + 1], sm.dyf[cell],
                          sm.dyf[cell + TX], src, sq);
     }
@@ -582,7 +587,7 @@ __device__ __forceinline__ void mixed_tile_compute(const MixedArgs &a, const Ctl
 // reference jumps are copied with cp.async while the halo is being loaded,
 // and the update's own-cell inputs are prefetched at the start of phase 3.
 template <int TX, int TY, int NT, int RS, bool BDF, bool PF = false>
-__device__ __forceinline__ void mixed_tile(const MixedArgs &a, const CtlHead<float> &head, int stage, float alpha, int bx,
+__device__ __forceinline__ void mixed_tile(const MixedArgs &a, const CtlHead<float> &head, int stage, float inv_alpha, int bx,
                                            int by, double *partial, unsigned char *smem_raw) {
     using S = MixedSmem<TX, TY>;
     static_assert((TX * TY) % NT == 0 && NT % 32 == 0, "tile/thread shape");
@@ -723,11 +728,11 @@ __device__ __forceinline__ void mixed_tile(const MixedArgs &a, const CtlHead<flo
         cp_async_wait_all();
         __syncthreads();
         PrefetchSrc src{a, d0, {}};
-        mixed_tile_compute<TX, TY, NT, RS, BDF, true>(a, head, stage, alpha, x0, y0, interior, partial, sm, src);
+        mixed_tile_compute<TX, TY, NT, RS, BDF, true>(a, head, stage, inv_alpha, x0, y0, interior, partial, sm, src);
     } else {
         __syncthreads();
         DirectSrc src{a, d0};
-        mixed_tile_compute<TX, TY, NT, RS, BDF, false>(a, head, stage, alpha, x0, y0, interior, partial, sm, src);
+        mixed_tile_compute<TX, TY, NT, RS, BDF, false>(a, head, stage, inv_alpha, x0, y0, interior, partial, sm, src);
     }
 }
 
@@ -739,7 +744,7 @@ stage_kernel_mixed(const MixedArgs a) {
     pdl_wait();
     const CtlHead<float> head = ctl_head<float>(a.ctl);
     if (head.done) return;
-    mixed_tile<TX, TY, NT, RS, BDF, PF>(a, head, a.stage, a.alpha, blockIdx.x, blockIdx.y,
+    mixed_tile<TX, TY, NT, RS, BDF, PF>(a, head, a.stage, a.inv_alpha, blockIdx.x, blockIdx.y,
                            a.partials + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * 4, smem_raw);
 }
 
@@ -780,7 +785,7 @@ struct StripRing {
     float4 e[4][32];   // dQ^{m}, dp^{m} (the ring terms)
     float jx[4][32];   // level jump across the east x-face (0 off the tank's rows)
     float jy[4][32];   // level jump across the south y-face (0 off the tank's faces)
-    float dt[4][32];   // local pseudo-time step that stage 1 stored (later stages, default options)
+    float dt[4][32];   // inverse of the local pseudo-time step, as stage 1 stored it (later stages, default options)
 };
 
 __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
@@ -806,7 +811,7 @@ struct HeldSrc {
     }
 };
 
-// One strip (strip coordinates sx, sy) of stage `stage` (coefficient alpha)
+// One strip (strip coordinates sx, sy) of stage `stage` (coefficient 1/inv_alpha)
 // of one tank, by one warp; `partial` receives the strip's four residual
 // partial sums at stage 1.  Shared by the single-tank and batched kernels.
 // The per-column parts of the boundary logic are formed once per strip and
@@ -826,7 +831,7 @@ struct HeldSrc {
 // windows reach ghost rows; the main loop then tests neither the row number
 // nor the fold of ghost rows.
 template <int H, int UNROLL = 1, int SK = 0>
-__device__ __forceinline__ void mixed_strip(const MixedArgs &a, const CtlHead<float> &head, int stage, float alpha, int sx,
+__device__ __forceinline__ void mixed_strip(const MixedArgs &a, const CtlHead<float> &head, int stage, float inv_alpha, int sx,
                                             int sy, double *partial, StripRing *ring) {
     constexpr bool FAST = SK != 0;
     const bool st1 = SK == 0 ? (stage == 1) : (SK == 1);
@@ -992,7 +997,7 @@ __device__ __forceinline__ void mixed_strip(const MixedArgs &a, const CtlHead<fl
                     // row k - 2 is a tank row, so its slot holds this column's records
                     const float4 ue = ering(s2), uq = ring->q[s2][lane];
                     const HeldSrc Uk{ue.x, ue.y, ue.z, ue.w, uq.x, uq.y, uq.z, uq.w};
-                    cell_update<false, FAST, SK>(a, alpha, inv_dt, b0dt, st1, dout, 0, (k - 2) * nx + c, Fw, Fxm2,
+                    cell_update<false, FAST, SK>(a, inv_alpha, inv_dt, b0dt, st1, dout, 0, (k - 2) * nx + c, Fw, Fxm2,
                                                  Fyp, Fy, hidx, hidy, jw, Jm2, Jyp, jy1, Uk, sq, out_lane,
                                                  SK == 2 ? ring->dt[s2][lane] : 0.0f);
                 }
@@ -1049,7 +1054,7 @@ sweep_kernel_mixed(const MixedArgs a, int strips_x, int nstrips) {
     const int warp = blockIdx.x * WPC + (threadIdx.x >> 5);
     if (warp >= nstrips) return;   // whole warps only
     const int sy = warp / strips_x, sx = warp - sy * strips_x;
-    mixed_strip<H, SK == 1 ? 1 : 2, SK>(a, head, a.stage, a.alpha, sx, sy, a.partials + (size_t)warp * 4,
+    mixed_strip<H, SK == 1 ? 1 : 2, SK>(a, head, a.stage, a.inv_alpha, sx, sy, a.partials + (size_t)warp * 4,
                       reinterpret_cast<StripRing *>(strip_smem) + (threadIdx.x >> 5));
 }
 
