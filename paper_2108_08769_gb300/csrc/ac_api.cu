@@ -427,6 +427,11 @@ constexpr MixedVariant kMixedVariants[] = {
     {28, 256, 128, 4, false, true}, {28, 64, 256, 2, false, true},
     // one 448-cell tile per SM on a 256x256 grid (a single wave of CTAs), with and without prefetching
     {32, 14, 448, 1, true}, {32, 14, 448, 1},
+    // shorter strips where longer ones leave the SMs short of warps: a warp's rows are one serial chain,
+    // so half the rows take little more than half the time (per iteration with 8, 16, 32 rows and the best
+    // tile: 512x512 39.3, 42.3, 61.7, 47.1 us; 1024x512 59.5, 58.0, 64.1, 77.4; 2048x2048 391, 310, 275, 543,
+    // where 64 rows take 252)
+    {28, 16, 128, 4, false, true}, {28, 8, 128, 4, false, true},
 };
 constexpr int kNumMixedVariants = sizeof(kMixedVariants) / sizeof(kMixedVariants[0]);
 
@@ -523,7 +528,9 @@ struct MixedBackend : Backend {
             case 18: return launch_sweep<256, 4, 4>(a, g, pdl, s);
             case 19: return launch_sweep<64, 8, 2>(a, g, pdl, s);
             case 20: return launch_mixed<32, 14, 448, 1, kOsher, false, true>(a, g, pdl, s);
-            default: return launch_mixed<32, 14, 448, 1>(a, g, pdl, s);
+            case 21: return launch_mixed<32, 14, 448, 1>(a, g, pdl, s);
+            case 22: return launch_sweep<16, 4, 4>(a, g, pdl, s);
+            default: return launch_sweep<8, 4, 4>(a, g, pdl, s);
         }
     }
 

@@ -255,6 +255,8 @@ constexpr Variant kVariants[] = {
     {28, 32, 128, false, true}, {28, 64, 128, false, true}, {28, 128, 128, false, true},
     // the same strips held to 3 CTAs per SM (room for the descriptor reads without spills)
     {28, 32, 128, false, true}, {28, 64, 128, false, true}, {28, 128, 128, false, true},
+    // shorter strips for batches that leave the SMs short of warps
+    {28, 16, 128, false, true},
 };
 constexpr int kNumVariants = sizeof(kVariants) / sizeof(kVariants[0]);
 
@@ -451,7 +453,8 @@ int stage_launch(ac_batch *b, cudaStream_t s, int stage, int v) {
         case 11: e = L.strips<128>(s); break;
         case 12: e = L.strips<32, 3>(s); break;
         case 13: e = L.strips<64, 3>(s); break;
-        default: e = L.strips<128, 3>(s); break;
+        case 14: e = L.strips<128, 3>(s); break;
+        default: e = L.strips<16>(s); break;
     }
     if (e != cudaSuccess) return fail(AC_ERR_CUDA, "batch stage launch failed: %s", cudaGetErrorString(e));
     return AC_OK;
