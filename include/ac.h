@@ -209,8 +209,9 @@ int ac_set_profiling(ac_ctx *ctx, int on);
 int ac_stage_kernel_time(const ac_ctx *ctx, double *total_ms, long long *launches);
 
 /* The stage-sweep variant the autotuner chose at the first physical step
- * (AC_ERR_STATE before it): tile width tx, height ty, threads per CTA and
- * the variant's index in the library's table.  Setting the environment
+ * (AC_ERR_STATE before it): tile width tx, height ty, threads per CTA
+ * that update cells (the FP64 sweep may run more, which share the other work)
+ * and the variant's index in the library's table.  Setting the environment
  * variable AC_TILE (mixed form) or AC_TILE_F64 (FP64) to an index before the
  * first step forces that variant.  The Bassi and Roe fluxes always run
  * variant 0, and so does BDF2/BDF3 in the mixed form; the mixed form's

@@ -73,7 +73,7 @@ int fail(int code, const char *fmt, ...) {
 // grid (sizes the residual partial sums).
 size_t max_tiles(int nx, int ny) {
     static const int shapes[][2] = {{32, 8}, {32, 7}, {32, 6}, {32, 4}, {16, 8}, {16, 16},
-                                    {32, 14}, {64, 7}, {32, 16}, {64, 8}, {64, 16}};
+                                    {32, 14}, {64, 7}, {8, 8}, {32, 16}, {64, 8}, {64, 16}};
     size_t m = 0;
     for (const auto &sh : shapes)
         m = std::max(m, (size_t)((nx + sh[0] - 1) / sh[0]) * ((ny + sh[1] - 1) / sh[1]));
@@ -162,15 +162,23 @@ const double kBDF[4][4] = {
 
 // ------------------------------------------------------------------ FP64
 
-// Tile shapes of the FP64 sweep (one thread per cell).  The FP64 pipe bounds
+// Tile shapes of the FP64 sweep (one thread per cell or more, f64_threads).  The FP64 pipe bounds
 // this sweep, so the shapes differ mainly in how evenly the CTAs fill the
 // SMs: small grids favour shapes whose CTA count is near a multiple of the
 // SM count.
 struct F64Variant {
     int tx, ty;
 };
-// 32x14 and 64x7 make one 448-cell tile per SM on a 256^2 grid (152 SMs)
-constexpr F64Variant kF64Variants[] = {{32, 8}, {32, 7}, {32, 6}, {32, 4}, {16, 8}, {16, 16}, {32, 14}, {64, 7}};
+// 32x14 and 64x7 make one 448-cell tile per SM on a 256^2 grid (152 SMs).
+// 8x8 is for grids that larger tiles leave most of the chip idle on: a stage
+// there lasts as long as one tile's chain of phases, and two threads per cell
+// of a 64-cell tile run the longest of them, the faces, in two passes
+// (pseudo-iterations of 200x4, 20x20, 64x64: 55, 56, 57 us on the best other
+// tile -> 33, 40, 41; 128x128 57 -> 54; 200x200 98 against 84).
+constexpr F64Variant kF64Variants[] = {{32, 8}, {32, 7}, {32, 6}, {32, 4}, {16, 8}, {16, 16}, {32, 14}, {64, 7}, {8, 8}};
+// Cells above which the 8x8 tile is not tried: two per SM fill the chip there
+// and its halo (144 cells loaded for 64) can only lose (table above)
+constexpr size_t kSmallTileCells = 2 * 152 * 64;
 constexpr int kNumF64Variants = sizeof(kF64Variants) / sizeof(kF64Variants[0]);
 
 template <int TX, int TY, int RS = kOsher>
@@ -198,7 +206,7 @@ struct F64Backend : Backend {
         const F64Variant &m = kF64Variants[variant < 0 ? 0 : variant];
         tx = m.tx;
         ty = m.ty;
-        nt = f64_threads(m.tx, m.ty);
+        nt = m.tx * m.ty;   // one per cell; f64_threads may add some that share the faces only
         return variant;
     }
 
@@ -225,7 +233,8 @@ struct F64Backend : Backend {
             case 4: e = launch_f64<16, 8>(a, g, pdl, s); break;
             case 5: e = launch_f64<16, 16>(a, g, pdl, s); break;
             case 6: e = launch_f64<32, 14>(a, g, pdl, s); break;
-            default: e = launch_f64<64, 7>(a, g, pdl, s); break;
+            case 7: e = launch_f64<64, 7>(a, g, pdl, s); break;
+            default: e = launch_f64<8, 8>(a, g, pdl, s); break;
         }
         if (e != cudaSuccess) return fail(AC_ERR_CUDA, "stage sweep launch failed: %s", cudaGetErrorString(e));
         return AC_OK;
@@ -260,6 +269,7 @@ struct F64Backend : Backend {
         const int S = c->opt.rk_stages;
         for (int pass = 0; pass < 2; ++pass)
             for (int v = 0; v < kNumF64Variants; ++v) {
+                if (kF64Variants[v].tx == 8 && c->N > kSmallTileCells) continue;
                 int rc;
                 // every stage of one pseudo-iteration (stages write only the two
                 // scratch buffers; the level Q^m is untouched)
@@ -331,6 +341,7 @@ struct F64Backend : Backend {
         CK((allow_f64_smem<16, 16>()));
         CK((allow_f64_smem<32, 14>()));
         CK((allow_f64_smem<64, 7>()));
+        CK((allow_f64_smem<8, 8>()));
         CK((allow_f64_smem<32, 8, kBassi>()));
         CK((allow_f64_smem<32, 8, kRoe>()));
         return AC_OK;

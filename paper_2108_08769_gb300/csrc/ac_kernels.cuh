@@ -280,8 +280,11 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 
 // Threads of the FP64 sweep's CTA on a TX x TY tile: one per cell, but 16 warps
 // on the 32x14 tile, whose two groups then have two warps on each of the four
-// SM sub-partitions (14 warps leave one warp alone on some).
-__host__ __device__ constexpr int f64_threads(int tx, int ty) { return tx == 32 && ty == 14 ? 512 : tx * ty; }
+// SM sub-partitions (14 warps leave one warp alone on some), and two per cell
+// on the 8x8 tile, whose faces then take two passes.
+__host__ __device__ constexpr int f64_threads(int tx, int ty) {
+    return tx == 32 && ty == 14 ? 512 : tx * ty == 64 ? 128 : tx * ty;
+}
 
 template <typename T, int TX, int TY>
 struct StageSmem {
@@ -343,6 +346,14 @@ stage_kernel(const SweepArgs<T> a) {
     const int nx = a.nx, ny = a.ny;
     const int tid = threadIdx.x;
     const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
+    // Rows of the tile inside the domain: tiles of under 256 cells load, slope
+    // and solve nothing for the rows past them (100x1: 55 -> 32 us per
+    // pseudo-iteration).  Larger tiles, picked only on grids of many rows,
+    // keep constant bounds: there the rows saved are few and the bounds' extra
+    // registers cost more (600x401 on 32x8: 297 -> 303 us, 256x256 on 32x14:
+    // 86.0 -> 86.7).
+    constexpr bool TRIM = TX * TY < 256;
+    const int th = TRIM ? min(TY, ny - y0) : TY;
 
     // A tile whose halo lies inside the domain needs no ghost folding.  The
     // ring's real-time inputs are loaded first and used last, and interior
@@ -359,7 +370,7 @@ stage_kernel(const SweepArgs<T> a) {
         for (int r = 0; r < NR; ++r) {
             const int k = tid + r * NT;
             rt_f[r] = 0;
-            if (k >= GW * GH) continue;
+            if (k >= GW * (th + 2)) continue;
             const int gi = x0 + (k % GW) - 1, gj = y0 + (k / GW) - 1;
             if (interior) {
                 rt_s[r] = gj * nx + gi;
@@ -405,7 +416,7 @@ stage_kernel(const SweepArgs<T> a) {
         for (int r = 0; r < NW; ++r)
             if (tid + r * NT < RW * RH) put_w(tid + r * NT, in4[r][0], in4[r][1], in4[r][2], in4[r][3]);
     } else {
-        for (int k = tid; k < RW * RH; k += NT) {
+        for (int k = tid; k < RW * (th + 4); k += NT) {
             const int gi = x0 + (k % RW) - 2, gj = y0 + (k / RW) - 2;
             int nfx, tfx, nfy, tfy;
             const int si = fold_axis(gi, nx, a.bc[0], a.bc[1], nfx, tfx);
@@ -422,7 +433,7 @@ stage_kernel(const SweepArgs<T> a) {
 #pragma unroll
         for (int r = 0; r < NR; ++r) {
             const int k = tid + r * NT;
-            if (k >= GW * GH) continue;
+            if (k >= GW * (th + 2)) continue;
             T rx = rt_q[r][0], ry = rt_q[r][1];
             if (!reuse_now) {
                 rx = realtime_term(a, rx, rt_l[r][0], 1, rt_s[r], inv_dt);
@@ -444,7 +455,9 @@ stage_kernel(const SweepArgs<T> a) {
     const int grp = GR == 2 ? tid / NTG : 0, tg = tid - grp * NTG;
     constexpr int R0 = GR == 2 ? TY / 2 + 2 : GH;      // ring rows the first group's faces need
     if (GR == 2 && grp == 1) bar_sync(3, NT);          // the first group's slopes first
-    for (int k = grp * (R0 * GW) + tg; k < (GR == 2 && grp == 0 ? R0 * GW : GW * GH); k += NTG) {
+    static_assert(!TRIM || GR == 1, "a trimmed tile works in one group");
+    const int kend = GR == 2 && grp == 0 ? R0 * GW : GW * (th + 2);
+    for (int k = grp * (R0 * GW) + tg; k < kend; k += NTG) {
         const int li = k % GW, lj = k / GW;            // ring coords (cell li-1, lj-1)
         const int c = (lj + 1) * RW + (li + 1);
         const int e = c + 1, wv = c - 1, nn = c + RW, ss = c - RW;
@@ -513,10 +526,14 @@ stage_kernel(const SweepArgs<T> a) {
     // The warps of a CTA sit on contiguous slots, so warps w and w + 4 share a
     // sub-partition; its share, faces [32 P s, 32 P (s + 1)) of the group's F,
     // P = ceil(F / 128), goes to its warps of the group in passes of 32, round-robin.
-    constexpr int NWG = NTG / 32, XG = S::NXF / GR;   // warps and x-faces of a group
+    // The faces of th rows are a prefix of each kind; on a grid of few rows
+    // they are one or two passes, not three.
+    constexpr int NWG = NTG / 32, HG = TY / GR;       // warps and rows of a group
     static_assert(NWG >= 4, "face schedule needs four warps");
-    const int yf0 = GR == 2 && grp == 1 ? (TY / 2 + 1) * TX : 0;                    // the group's first y-face
-    const int yfn = GR == 2 ? (grp == 0 ? (TY / 2 + 1) * TX : (TY / 2) * TX) : S::NYF;   // and their number
+    const int rows = TRIM ? th : HG;                               // the group's rows
+    const int XG = rows * (TX + 1), xf0 = grp * (HG * (TX + 1));   // its x-faces and the first of them
+    const int yf0 = grp * ((HG + 1) * TX);                         // its first y-face and their number: the first
+    const int yfn = (grp == 0 ? rows + 1 : rows) * TX;             // group takes the faces between the groups
     const int nf = XG + yfn, fp = (nf + 127) / 128;
     const int fw = tid >> 5, sub = fw & 3;
     const int w0 = grp * NWG + ((sub - grp * NWG) & 3);            // the sub-partition's first warp of the group
@@ -525,7 +542,7 @@ stage_kernel(const SweepArgs<T> a) {
     for (int fq = (fw - w0) >> 2; fbeg + 32 * fq < fend; fq += fwarps) {
         const int kf = fbeg + 32 * fq + (tid & 31);
         if (kf >= fend) continue;
-        const int k = kf < XG ? grp * XG + kf : S::NXF + yf0 + (kf - XG);
+        const int k = kf < XG ? xf0 + kf : S::NXF + yf0 + (kf - XG);
         const bool isx = k < S::NXF;
         // face states: density, normal and tangential velocity (rotation,
         // Alg. 2: (u, v) on x-faces, (v, u) on y-faces), pressure
