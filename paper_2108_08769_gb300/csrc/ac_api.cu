@@ -838,11 +838,7 @@ int enqueue_iteration(ac_ctx *c, cudaStream_t s, unsigned long long cond, int us
     if (!c->opt.local_dtau && (rc = c->be->dtau_min(c, s)) != AC_OK) return rc;
     if (timed) CK(cudaEventRecord(c->ev[0], s));
     for (int st = 1; st <= c->opt.rk_stages; ++st) {
-        // An iteration's first stage waits for the end of the one before to
-        // drain: launched with a programmatic dependency, the CTAs of a strip
-        // sweep that fills the SMs took 84 instead of 65 us per iteration on
-        // 1024x512 cells; small grids lose nothing.
-        if ((rc = c->be->stage(c, s, st, c->pdl && st > 1)) != AC_OK) return rc;
+        if ((rc = c->be->stage(c, s, st, c->pdl)) != AC_OK) return rc;
         if (timed) CK(cudaEventRecord(c->ev[st], s));
     }
     CK(launch_pdl(c->pdl, end_iteration_kernel, dim3(1), dim3(kEndLanes), 0, s, c->ctl, c->partials, e));

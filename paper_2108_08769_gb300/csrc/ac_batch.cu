@@ -72,8 +72,8 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 3 : 6)
 batch_stage_kernel(const BatchTank *__restrict__ tanks, const int *__restrict__ tile_tank, int stage, float inv_alpha,
                    int slot0) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const int k = tile_tank[blockIdx.x];
     if constexpr (CD) {
         const BatchTank &t = c_tanks[slot0 + k];
@@ -101,8 +101,8 @@ batch_sweep_kernel(const BatchTank *__restrict__ tanks, const int *__restrict__ 
                    float inv_alpha, int slot0) {
     extern __shared__ __align__(16) unsigned char strip_smem[];
     StripRing *ring = reinterpret_cast<StripRing *>(strip_smem) + (threadIdx.x >> 5);
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const int w = blockIdx.x * WPC + (threadIdx.x >> 5);
     if (w >= nstrips) return;   // whole warps only
     const int k = strip_tank[w];
@@ -166,8 +166,8 @@ __global__ void batch_jumps_kernel(const BatchTank *tanks) {
 // end of iteration asked for one (blockIdx.y = tank); the jumps follow in a
 // second launch.
 __global__ void batch_rebase_shift_kernel(const BatchTank *tanks) {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const MixedArgs &a = tanks[blockIdx.y].a;
     if (!a.ctl->rebase) return;
     const int cur = a.ctl->cur;
@@ -177,8 +177,8 @@ __global__ void batch_rebase_shift_kernel(const BatchTank *tanks) {
 }
 
 __global__ void batch_rebase_jumps_kernel(const BatchTank *tanks) {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const MixedArgs &a = tanks[blockIdx.y].a;
     if (!a.ctl->rebase) return;
     const size_t N = (size_t)a.nx * a.ny;
@@ -195,8 +195,8 @@ __global__ void __launch_bounds__(NT)
 batch_end_kernel(BatchTank *tanks, BatchSync *sync, int ntanks, unsigned long long cond, int use_cond) {
     static_assert(NT >= kEndLanes, "sum_partials_fixed needs kEndLanes threads");
     const int tid = threadIdx.x;
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const BatchTank &t = tanks[blockIdx.x];
     Ctl *ctl = t.a.ctl;
     const bool was_done = ctl->done != 0;
@@ -509,13 +509,9 @@ int tune(ac_batch *b, cudaStream_t s) {
 // One pseudo-iteration; rebase adds the kernels that act after iterations 1, 2, 4, 8.
 int enqueue_iteration(ac_batch *b, cudaStream_t s, unsigned long long cond, int use_cond, bool timed, bool rebase) {
     int rc;
-    const bool pdl = b->pdl;
     if (timed) CK(cudaEventRecord(b->ev[0], s));
     for (int st = 1; st <= b->opt.rk_stages; ++st) {
-        b->pdl = pdl && st > 1;   // the first stage waits for the iteration before to drain (see ac_api.cu)
-        rc = stage_launch(b, s, st, b->variant);
-        b->pdl = pdl;
-        if (rc != AC_OK) return rc;
+        if ((rc = stage_launch(b, s, st, b->variant)) != AC_OK) return rc;
         if (timed) CK(cudaEventRecord(b->ev[st], s));
     }
     CK(launch_pdl(b->pdl, batch_end_kernel<256>, dim3(b->n), dim3(256), 0, s, b->tanks_dev, b->sync, b->n, cond,

@@ -274,7 +274,12 @@ __device__ __forceinline__ T wall_ghost_sign(int gi, int gj, int nx, int ny, con
 // Programmatic dependent launch: let the next kernel in the stream be
 // scheduled (its CTAs then wait in pdl_wait), and wait until the previous
 // kernel has finished and its writes are visible.  No-ops for a kernel
-// launched without the programmatic-serialization attribute.
+// launched without the programmatic-serialization attribute.  Every kernel
+// waits first and triggers then: CTAs that triggered before their wait let the
+// kernel after them in as well, and the waiting CTAs of two kernels filled the
+// SMs' free slots unevenly (per iteration, trigger first -> wait first:
+// 256x256 mixed tiles 26.9 -> 26.0 us, 1024x512 in 16-row strips 57.8 -> 54.8,
+// 1024x1024 in 32-row strips 93.1 -> 84.5; FP64 and larger grids as before).
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -330,8 +335,8 @@ stage_kernel(const SweepArgs<T> a) {
     // beside the second's faces (256x256 tank: 105 -> 91 us per pseudo-iteration).
     constexpr int GR = (TX == 32 && TY == 14) ? 2 : 1, NTG = NT / GR;
 
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const Ctl *ctl = a.ctl;
     const CtlHead<T> head = ctl_head<T>(ctl);
     if (head.done) return;
@@ -705,8 +710,8 @@ stage_kernel(const SweepArgs<T> a) {
 // (Sec. 2.2.3), from Q^{m}.  Positive doubles order like their bit patterns.
 template <typename T>
 __global__ void dtau_min_kernel(const SweepArgs<T> a) {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const Ctl *ctl = a.ctl;
     if (ctl->done) return;
     const T *const *q = a.buf[ctl->cur];
@@ -780,8 +785,8 @@ __global__ void begin_step_kernel(const SweepArgs<T> a, double dt, double tol, i
 // while-condition when launched inside a captured loop.
 static __global__ void __launch_bounds__(kEndLanes)
 end_iteration_kernel(Ctl *ctl, const double *partials, const IterEnd e) {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     if (ctl->done) {
         if (e.use_cond && threadIdx.x == 0) cudaGraphSetConditional(e.cond, 0);
         return;

@@ -740,8 +740,8 @@ template <int TX, int TY, int NT, int MINB = 1, int RS = kOsher, bool BDF = fals
 __global__ void __launch_bounds__(NT, MINB)
 stage_kernel_mixed(const MixedArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const CtlHead<float> head = ctl_head<float>(a.ctl);
     if (head.done) return;
     mixed_tile<TX, TY, NT, RS, BDF, PF>(a, head, a.stage, a.inv_alpha, blockIdx.x, blockIdx.y,
@@ -1046,8 +1046,8 @@ __device__ __forceinline__ void mixed_strip(const MixedArgs &a, const CtlHead<fl
 template <int H, int WPC, int MINB, int SK>
 __global__ void __launch_bounds__(WPC * 32, MINB)
 sweep_kernel_mixed(const MixedArgs a, int strips_x, int nstrips) {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const CtlHead<float> head = ctl_head<float>(a.ctl);
     if (head.done) return;
     extern __shared__ __align__(16) unsigned char strip_smem[];
@@ -1060,8 +1060,8 @@ sweep_kernel_mixed(const MixedArgs a, int strips_x, int nstrips) {
 
 // Global pseudo-time step option for the mixed form.
 static __global__ void dtau_min_kernel_mixed(const MixedArgs a) {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const Ctl *ctl = a.ctl;
     if (ctl->done) return;
     const float4 *d = a.d[ctl->cur];
@@ -1209,8 +1209,8 @@ __device__ __forceinline__ void mixed_rebase_shift(const MixedArgs &a, int cur, 
 // The end of iteration m sets ctl->rebase after m = 1, 2, 4, 8 (not on the
 // last iteration); otherwise these return at once.
 static __global__ void rebase_shift_kernel_mixed(const MixedArgs a) {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const Ctl *ctl = a.ctl;
     if (!ctl->rebase) return;
     const int cur = ctl->cur;
@@ -1220,8 +1220,8 @@ static __global__ void rebase_shift_kernel_mixed(const MixedArgs a) {
 }
 
 static __global__ void rebase_jumps_kernel_mixed(const MixedArgs a) {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     if (!a.ctl->rebase) return;
     const size_t N = (size_t)a.nx * a.ny;
     for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < N; g += (size_t)gridDim.x * blockDim.x)
