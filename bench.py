@@ -353,7 +353,8 @@ def run_ours(args, ws, rank, local):
                 "kernel": f"stage_kernel<double,{ftx},{fty}>", "tile_variant": fv,
                 "launch_ms": per_launch_s * 1e3, "launch_ms_timed_alone": isolated_s * 1e3,
                 "flops_per_cell_stage": FP64_ALG_FLOPS_PER_CELL_STAGE,
-                "flops_note": "algorithmic FP64 flops of one stage per cell, fixed (derivation in the design notes)",
+                "flops_note": "algorithmic FP64 flops of one stage per cell, fixed (derivation in the design notes); the fluxes' 356 "
+                              "of them run in block fixed point on the integer pipes, beside the FP64 unit",
                 "executed_flops_per_cell_stage": FP64_EXEC_FLOPS_PER_CELL_STAGE,
                 "executed_frac": FP64_EXEC_FLOPS_PER_CELL_STAGE * case.cells / per_launch_s / 1e12 / FP64_PEAK_TFLOPS,
                 "peak_source": "nominal FP64 rate of the part (profiling recipe: 2 FP64 FMA lanes/SM)",
@@ -619,16 +620,16 @@ def run_batched(args, stream, flush, barrier):
 # move when the kernel executes fewer or more operations (recomputation on
 # a tile's ring, stage-1 values read back), only with the formulation.
 FP64_ALG_FLOPS_PER_CELL_STAGE = 483.0
-# what stage_kernel<double,32,14> executes on this 256x256 tank (ncu: DFMA x 2
-# + DADD + DMUL, mean of stages 1-3: 721.2, 639.2, 639.2; the tile's ring
-# recomputes slopes and pressure gradients, and stage 1 forms the values
-# stages 2 and 3 read back), and the FP64 instructions behind them
-FP64_EXEC_FLOPS_PER_CELL_STAGE = 666.5
-FP64_INSTR_PER_CELL_STAGE = 455.3
+# what stage_kernel<double,32,14>'s FP64 unit executes on this 256x256 tank
+# (ncu: DFMA x 2 + DADD + DMUL, mean of stages 1-3: 173.7, 143.4, 143.4; the
+# fluxes' 356 flops run on the integer pipes), and the FP64 instructions
+# behind them
+FP64_EXEC_FLOPS_PER_CELL_STAGE = 153.5
+FP64_INSTR_PER_CELL_STAGE = 112.9
 FP64_PIPE_INSTR_PER_S = 2 * 152 * 2.07e9
 # DRAM bytes per cell of one FP64 stage launch, same capture, averaged over
-# the three stages (3.74, 6.36, 6.36 MB read; the output stays in L2)
-FP64_TRAFFIC_PER_CELL_STAGE = 83.7
+# the three stages (3.77, 6.38, 6.38 MB read; the output stays in L2)
+FP64_TRAFFIC_PER_CELL_STAGE = 84.1
 # algorithmic HBM bytes per cell-iteration of the FP64 sweep (s_max = 3):
 # stage 1 reads Q^{m} (32 B) and Q^n (24 B), writes Q^1 (32 B) and the four
 # per-cell values kept for the later stages (32 B); stages 2 and 3 read
@@ -637,7 +638,7 @@ BYTES_PER_CELL_ITER_F64 = 376.0
 # mixed form: stage 1 reads the (Q^n, rho_ref) and (dQ^{m}, dp^{m}) records
 # (2 x 16 B) and the level-jump record (8 B) and writes 16 B; stages 2 and 3
 # also read the (dQ^{s-1}, dp^{s-1}) record (16 B).  The column-strip sweep
-# moves 4 B per cell and stage more (stage 1 stores the local pseudo-time
+# moves 4 B per cell and stage more (stage 1 stores the inverse local pseudo-time
 # step, stages 2 and 3 read it): 212 B, a choice of the kernel, not counted here
 MIXED_BYTES_PER_CELL_ITER = 56.0 + 2 * 72.0
 # measured (ncu, stages 1 and 2 of a pseudo-iteration on this 2048x8192
@@ -647,8 +648,8 @@ MIXED_BYTES_PER_CELL_ITER = 56.0 + 2 * 72.0
 # mean over the three stages (stage 3 as stage 2).  A variant without a
 # capture of its current code reports null.
 MIXED_COUNTS_BY_VARIANT = {
-    16: ((61.5 + 2 * 79.7) / 3, (449.7 + 2 * 405.6) / 3),   # sweep_kernel_mixed<64,4,4,1>, <64,4,4,2>
-    17: ((60.0 + 2 * 77.5) / 3, (446.5 + 2 * 402.4) / 3),   # sweep_kernel_mixed<128,4,4,1>, <128,4,4,2>
+    16: ((61.5 + 2 * 79.7) / 3, (394.0 + 2 * 359.1) / 3),   # sweep_kernel_mixed<64,4,4,1>, <64,4,4,2>
+    17: ((60.0 + 2 * 77.5) / 3, (390.8 + 2 * 356.0) / 3),   # sweep_kernel_mixed<128,4,4,1>, <128,4,4,2>
 }
 FP32_PEAK_TOPS = 128 * 152 * 2.07e9 / 1e12
 

@@ -162,9 +162,10 @@ const double kBDF[4][4] = {
 
 // ------------------------------------------------------------------ FP64
 
-// Tile shapes of the FP64 sweep (one thread per cell or more, f64_threads).  The FP64 pipe bounds
-// this sweep, so the shapes differ mainly in how evenly the CTAs fill the
-// SMs: small grids favour shapes whose CTA count is near a multiple of the
+// Tile shapes of the FP64 sweep (one thread per cell or more, f64_threads).
+// Arithmetic (the integer pipes for the fluxes, the FP64 unit for the rest)
+// bounds this sweep, so the shapes differ mainly in how evenly the CTAs fill
+// the SMs: small grids favour shapes whose CTA count is near a multiple of the
 // SM count.
 struct F64Variant {
     int tx, ty;
@@ -301,7 +302,6 @@ struct F64Backend : Backend {
         a.riemann = c->opt.riemann;
         a.local_dtau = c->opt.local_dtau; a.alpha_pi_p_row = c->opt.alpha_pi_p_row;
         a.stage = stage; a.s_max = c->opt.rk_stages;
-        a.alpha = stage > 0 ? 1.0 / double(c->opt.rk_stages - stage + 1) : 0.0;
         const double dx = c->dx, dy = c->dy;
         a.dx = dx; a.dy = dy; a.half_dx = 0.5 * dx; a.half_dy = 0.5 * dy;
         a.inv_dx = 1.0 / dx; a.inv_dy = 1.0 / dy; a.dx_over_dy = dx / dy; a.dy_over_dx = dy / dx;
@@ -440,7 +440,7 @@ constexpr MixedVariant kMixedVariants[] = {
     {32, 14, 448, 1, true}, {32, 14, 448, 1},
     // shorter strips where longer ones leave the SMs short of warps: a warp's rows are one serial chain,
     // so half the rows take little more than half the time (per iteration with 8, 16, 32 rows and the best
-    // tile: 512x512 39.3, 42.3, 61.7, 47.1 us; 1024x512 59.5, 58.0, 64.1, 77.4; 2048x2048 391, 310, 275, 543,
+    // tile: 512x512 39.3, 42.3, 61.7, 47.1 us; 1024x512 59.5, 54.9, 63.7, 77.4; 2048x2048 391, 310, 275, 543,
     // where 64 rows take 252)
     {28, 16, 128, 4, false, true}, {28, 8, 128, 4, false, true},
 };
@@ -485,7 +485,7 @@ struct MixedBackend : Backend {
     float4 *d[3] = {};   // per cell (dQ of rho, rho u, rho v; dp or p), three rotating buffers
     float4 *qn = nullptr;  // per cell (FP32 Q^n of rho, rho u, rho v; rho_ref)
     float2 *jmp = nullptr;   // per cell level jumps (west face, south face)
-    float *dtau = nullptr;   // per cell local pseudo-time step (column-strip sweep, default options)
+    float *dtau = nullptr;   // per cell inverse local pseudo-time step (column-strip sweep, default options)
     float *lev_p = nullptr;
     float *D1[3] = {}, *D2[3] = {};   // Q^n - Q^{n-1}, Q^n - Q^{n-2} (BDF2, BDF3)
     double *q64[4] = {};   // FP64 levels of rho, rho u, rho v, p

@@ -342,7 +342,7 @@ struct ac_batch {
     float4 *qn;                         // per cell (FP32 Q^n of rho, rho u, rho v; rho_ref)
     float2 *jmp;                        // per cell level jumps (west face, south face)
     float *lev_p;                       // restore copy of p (without a level)
-    float *dtau;                        // local pseudo-time steps (column-strip sweep, default options)
+    float *dtau;                        // inverse local pseudo-time steps (column-strip sweep, default options)
     float *D1[3], *D2[3];               // BDF2/BDF3 level differences (pools)
     double *q64[4];                     // FP64 levels of rho, rho u, rho v, p
     double *p64_step;                   // FP64 pressure levels at the start of the step

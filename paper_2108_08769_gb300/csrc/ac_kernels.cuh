@@ -87,7 +87,6 @@ struct SweepArgs {
     int gradp, limiter_k, realtime, local_dtau, alpha_pi_p_row;
     int riemann;                   // kOsher / kBassi / kRoe
     int stage, s_max;
-    T alpha;                       // alpha_s of this stage
     T dx, dy, half_dx, half_dy, inv_dx, inv_dy, dx_over_dy, dy_over_dx;
     T beta, inv_beta, gx, gy;
     int fixed;                     // the Osher flux may run in fixed point (beta and the cell sizes allow it)
@@ -104,14 +103,14 @@ struct SweepArgs {
     double *partials;              // per-CTA residual partial sums [nblocks][4]
     Ctl *ctl;
     // Per-cell values that stay fixed through a pseudo-iteration (they come
-    // from Q^{m} and the real-time levels): local dtau and the real-time
+    // from Q^{m} and the real-time levels): 1/dtau (local) and the real-time
     // terms of rho, rho u, rho v.  With reuse set, stage 1 writes them and
     // later stages read them back instead of recomputing; null otherwise.
     T *aux[4];
     int reuse;
 };
 
-// The constants of the fixed-point flux and of the scaled fluxes; alpha and cfl_area are set.
+// The constants of the fixed-point flux and of the scaled fluxes; stage, s_max and cfl_area are set.
 inline void set_flux_scales(SweepArgs<double> &a, double beta, double dx, double dy) {
     a.fixed = fixed_beta_ok(beta) && fixed_beta_ok(dx) && fixed_beta_ok(dy);
     a.fbeta = make_fixed_beta(beta);
@@ -332,7 +331,8 @@ stage_kernel(const SweepArgs<T> a) {
     // while its faces keep the integer pipes busy.  Its warps therefore work in
     // two groups, one per half of the rows, the second a phase behind: the
     // first group's faces run beside the second's slopes, and its update
-    // beside the second's faces (256x256 tank: 105 -> 91 us per pseudo-iteration).
+    // beside the second's faces (256x256 tank: 105 -> 91 us per pseudo-iteration;
+    // 87 with what is now done less between the stages).
     constexpr int GR = (TX == 32 && TY == 14) ? 2 : 1, NTG = NT / GR;
 
     pdl_wait();

@@ -163,7 +163,6 @@ extern "C" int ac_stage_sweep_noalloc(const ac_grid *grid, double beta, const ac
     a.riemann = opt->riemann;
     a.local_dtau = opt->local_dtau ? 1 : 0; a.alpha_pi_p_row = opt->alpha_pi_p_row ? 1 : 0;
     a.stage = stage; a.s_max = opt->rk_stages;
-    a.alpha = 1.0 / double(opt->rk_stages - stage + 1);
     const double dx = grid->lx / grid->nx, dy = grid->ly / grid->ny;
     a.dx = dx; a.dy = dy; a.half_dx = 0.5 * dx; a.half_dy = 0.5 * dy;
     a.inv_dx = 1.0 / dx; a.inv_dy = 1.0 / dy; a.dx_over_dy = dx / dy; a.dy_over_dx = dy / dx;
