@@ -40,6 +40,7 @@ namespace acgb {
 struct FixedBeta {
     uint64_t b8, ib4, tib4;   // ib4: 8/9 of 1/(4 beta) (see fx::k89); tib4: sqrt(3/5)/2 times it, at the same exponent
     int eb8, eib4;
+    uint32_t most;            // most of rho u^2, as in fixed_flux_ok
 };
 
 // A positive factor of the returned flux as (63-bit mantissa in [2^62, 2^63), exponent).
@@ -64,6 +65,10 @@ inline FixedBeta make_fixed_beta(double beta) {
     f.ib4 = (uint64_t)((((unsigned __int128)1 << 127) / 9 * 2) / mant);
     f.eib4 = 61 - e - 125;
     f.tib4 = (uint64_t)(((unsigned __int128)f.ib4 * 7144393258922745604ull) >> 64);
+    const double b16 = 16.0 * beta;
+    uint64_t u;
+    memcpy(&u, &b16, 8);
+    f.most = (uint32_t)(u >> 32) + ((2u * 1023u) << 20);    // high word of 16 beta, biased as those of rho and twice u
     return f;
 }
 
@@ -313,7 +318,7 @@ struct Point {
 // Osher flux of one face (Dumbser and Toro, 3 Gauss points on the straight
 // path in Q): 2F = (mass, normal momentum, tangential momentum, p/beta flux),
 // returned times sc, the last component times scp; inputs as osher_flux.
-// Requires finite inputs and normal positive densities (fixed_flux_ok).
+// Requires states that fixed_flux_ok accepts.
 //
 // |A| has the eigenvalues u (three times) and (u +- c)/2 of opposite signs,
 // so with sg = sign(u) it is sg A + 2 |l| r l^T, rank one beside A itself, l
@@ -479,6 +484,21 @@ ACFX bool fixed_flux_ok(double rL, double uL, double vL, double pL, double rR, d
     auto m = [](double x) { return (uint32_t)(bits_of(x) >> 32) & 0x7fffffffu; };
     auto max2 = [](uint32_t a, uint32_t b) { return a > b ? a : b; };
     return max2(rl, rr) < most - lo && max2(max2(max2(m(uL), m(uR)), max2(m(vL), m(vR))), max2(m(pL), m(pR))) < most;
+}
+// And whether it may run on them: besides the range, rho u^2/(4 beta) at most 4 or so on both sides.  1 - |u|/c is a
+// difference of nearly equal terms where that ratio is large (an outer Gauss point's is at most 9 times the sides'
+// larger one).  From 16 on the flux of p/beta is further off than in FP64 (rms in units of 2^-53 of its terms: 0.7
+// and 1.3 at a ratio of 2 to 4, 3.6 and 3.0 at 16 to 32, 820 and 540 at 2^12).  The high words of doubles serve as
+// their logarithms (0.09 low at most), so that the limit lies between 4.0 and 4.8.  beta is mostly rho c0^2 with c0
+// ten times the velocities, and the ratio below 0.01.
+ACFX bool fixed_flux_ok(double rL, double uL, double vL, double pL, double rR, double uR, double vR, double pR,
+                        const FixedBeta &fb) {
+    using namespace fx;
+    auto q = [](double r, double u) {   // below 2^32 within the range
+        return (uint32_t)(bits_of(r) >> 32) + 2u * ((uint32_t)(bits_of(u) >> 32) & 0x7fffffffu);
+    };
+    const uint32_t ql = q(rL, uL), qr = q(rR, uR);
+    return fixed_flux_ok(rL, uL, vL, pL, rR, uR, vR, pR) && (ql > qr ? ql : qr) <= fb.most;
 }
 // The same for beta and the factors of the returned flux.
 inline bool fixed_beta_ok(double beta) { return beta > 1e-70 && beta < 1e70; }

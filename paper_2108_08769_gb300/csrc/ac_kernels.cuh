@@ -577,7 +577,7 @@ stage_kernel(const SweepArgs<T> a) {
         // Fluxes are stored as F/dx or F/dy (formed as 2F times 1/(2 dx)), the
         // pressure row times beta, so that the divergence is sums only.
         T F[4];
-        if (RS == kOsher && a.fixed && fixed_flux_ok(rL, nL, tL, pL, rR, nR, tR, pR)) {
+        if (RS == kOsher && a.fixed && fixed_flux_ok(rL, nL, tL, pL, rR, nR, tR, pR, a.fbeta)) {
             osher_flux_fixed(rL, nL, tL, pL, rR, nR, tR, pR, a.fbeta, isx ? a.fhx : a.fhy, isx ? a.fphx : a.fphy, F);
         } else {
             riemann_flux<RS, T, true>(rL, nL, tL, pL, rR, nR, tR, pR, a.beta, a.inv_beta, F);
