@@ -358,14 +358,16 @@ ACFX void osher_flux_fixed(double rLd, double uLd, double vLd, double pLd, doubl
     // jumps of p and u as signs and magnitudes in [2^61, 2^62); the point sums below are formed times sd = sign(du)
     const int sd = (int)(DU >> 63), sp = (int)(DPs >> 63) ^ sd;
     uint64_t DP = mag(DPs), du = mag(DU);
-    const int kd = room(DP), ku = room(du), epd = ep - kd;
+    // a zero jump's exponent is below all others, so that no common exponent is formed for its sake
+    const int none = -16384;
+    const int kd = room(DP), ku = room(du), epd = DP == 0 ? none : ep - kd;
     DP <<= kd;
     du <<= ku;
     // 2 rho_L rho_R |du| in [2^62, 2^63) (or 0)
     uint64_t D = mulu(mulu(rL.m, rR.m) * 2, du * 2);     // [2^59, 2^62)
     const int kD = clz32((uint32_t)(D >> 32) | 1u) - 1;
     D <<= kD;
-    int eb = rL.e + rR.e + (ed - ku) + 128 - kD - er;
+    int eb = du == 0 ? none : rL.e + rR.e + (ed - ku) + 128 - kD - er;
     // ---- first loop: u, c, a, b at the Gauss points (twice the states: r' = rS -+ t dr, m' = c0 -+ t dm) ----
     const int64_t TR = neg_if((int64_t)mulhi(kT64, mag(DR)), (int)(DR >> 63));
     const int64_t TM = neg_if((int64_t)mulhi(kT64, mag(DM)), (int)(DM >> 63));
@@ -445,8 +447,8 @@ ACFX void osher_flux_fixed(double rLd, double uLd, double vLd, double pLd, doubl
     int64_t ZV = neg_if(smul(fb.ib4, SZ), sd);
     int ez = ecx + eg + 126 + fb.eib4;
     const int nz = room(mag(ZV) | mag(TZ));
-    ZV <<= nz;
-    TZ <<= nz;
+    ZV = (int64_t)((uint64_t)ZV << nz);
+    TZ = (int64_t)((uint64_t)TZ << nz);
     ez -= nz;
     const int ev = imax(eu, ez) + 1;
     const int64_t S1 = (int64_t)shr(SU, ev - eu) + sar(TZ, ev - ez), Zv = sar(ZV, ev - ez);   // |.| < 2^62

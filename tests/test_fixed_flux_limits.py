@@ -100,3 +100,18 @@ def test_exponents_at_the_limits(lib):
         if max(abs(x) for x in v) < 2.0 ** 250:
             took += check(lib, [rL, u[0], v[0], p[0], rR, u[1], v[1], p[1]], beta)
     assert took > 300
+
+
+def test_equal_pressures_or_velocities_hide_nothing(lib):
+    """A jump that is exactly zero has no size: the other one keeps its bits beside it, whatever the pressures or
+    velocities themselves are (flow that has all but come to rest under a large head)."""
+    rng = np.random.default_rng(5)
+    for k in range(300):
+        rL, rR, beta = 10 ** rng.uniform(0, 3), 10 ** rng.uniform(0, 3), 10 ** rng.uniform(0, 6)
+        c = np.sqrt(beta / max(rL, rR))
+        p = beta * 10 ** rng.uniform(0, 12) * rng.choice([-1, 1])
+        u = c * 10 ** -rng.uniform(5, 40)
+        uR = [0.0, -u, 0.3 * u][k % 3]
+        assert check(lib, [rL, u, u * rng.normal(), p, rR, uR, u * rng.normal(), p], beta)
+        dp = beta * 10 ** -rng.uniform(10, 40)
+        assert check(lib, [rL, u, c * rng.normal(), dp, rR, u, c * rng.normal(), -dp], beta)
