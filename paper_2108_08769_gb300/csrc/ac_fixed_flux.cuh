@@ -1,19 +1,22 @@
 // ac_fixed_flux.cuh -- the Osher flux of the FP64 sweep, and FP64
 // reciprocals and square roots, on the integer pipes.
 //
-// GB300's FP64 unit takes 64 cycles per warp instruction and sub-partition,
-// while 64-bit integer adds, shifts and 64-bit high products take about 2, 4
-// and 14 and run beside it.  So the flux, three quarters of the FP64 sweep's
-// work, is evaluated in block fixed point: every quantity is a 64-bit integer
-// with at least 56 significant bits and a binary exponent of its own or of
-// its face (FP64 keeps 53), and the sweep's other arithmetic keeps the FP64
-// unit busy meanwhile.  A flux takes about 1770 instructions (2900 cycles per
-// warp with four warps on a sub-partition, near the integer multiplier's rate)
-// where the FP64 form took about 150 FP64 instructions, 10,000 cycles.  One
-// pseudo-iteration of the 256x256 tank: 193 -> 87 us, of a 1024x512 tank
-// 1440 -> 563 us (with the rest of the sweep thinned out to match, see
-// stage_kernel).  The FP64 unit is then busy 42-44 % of the cycles, not 80 %.  The error of 2F against 113-bit arithmetic, in units of 2^-53
-// of its terms, is 0.3-0.9 rms where the FP64 formula's is 0.7-1.7.
+// GB300's FP64 unit takes 16 cycles per warp instruction (one unit an SM, so
+// each of the four sub-partitions gets a turn every 64), while 64-bit integer
+// adds, shifts and 64-bit high products take a sub-partition about 2, 4 and 14
+// and run beside it.  So the flux, three quarters of the FP64 sweep's work, is
+// evaluated in block fixed point: every quantity is a 64-bit integer and a
+// binary exponent of its own or of the face's largest term of its kind, 56 bits
+// or more of that term (FP64 keeps 53), and the sweep's other arithmetic keeps
+// the FP64 unit busy meanwhile.  A flux takes about 1770 instructions (2900
+// cycles per warp with four warps on a sub-partition, near the integer
+// multiplier's rate) where the FP64 form took about 150 FP64 instructions,
+// 10,000 cycles.  One pseudo-iteration of the 256x256 tank: 193 -> 87 us, of a
+// 1024x512 tank 1440 -> 563 us (with the rest of the sweep thinned out to
+// match, see stage_kernel); the FP64 unit is then busy 42-44 % of the cycles,
+// not 80 %.  The error of 2F against 113-bit arithmetic, in units of 2^-53 of
+// its terms, is 0.3-0.9 rms where the FP64 formula's is 0.7-1.7, over the faces
+// that fixed_flux_ok accepts.
 //
 // A value is the pair (int, E): int 2^E.  "Q61" and the like: a number in
 // [0, 1] scaled by 2^61.
@@ -328,8 +331,9 @@ struct Point {
 // b = c rho_L rho_R (u_R - u_L) / rho, that is
 //   |A| dQ = |u| dQ' + (r Z, m Z + G, n Z, Z - u (G - sg dp)/beta),
 //   G = s b/2 + sg a dp,   Z = c (2 s dp + sg h b) / (4 beta),
-// dQ' = (d rho, d(rho u), d(rho v), 0): no difference of nearly equal terms
-// is left, and every factor but c, u, b and dp lies in [0, 1].  With
+// dQ' = (d rho, d(rho u), d(rho v), 0): the one difference of terms that may
+// be nearly equal is 1 - a (fixed_flux_ok bounds a), and every factor but c, u,
+// b and dp lies in [0, 1].  With
 // r_j = (rS -+ t dr)/2 and so on, sums over the points of r Z need only the
 // sum of Z and the difference of the outer points' Z.
 ACFX void osher_flux_fixed(double rLd, double uLd, double vLd, double pLd, double rRd, double uRd, double vRd,
