@@ -159,8 +159,8 @@ ACFX uint64_t bits_of(double x) {
 #endif
 }
 
-// A double as sign, 63-bit mantissa in [2^62, 2^63) and exponent.  Zero and subnormals become numbers near 2^-1022,
-// which vanish beside any normal number and which to_double makes zero again.
+// A double as sign, 63-bit mantissa in [2^62, 2^63) and exponent.  Zeros and subnormals have no mantissa: a number
+// near 2^-1022 instead would leave -1 behind where a negative one is shifted far to the right.
 struct Num {
     uint64_t m;
     int e, s;   // s = -1 for a negative number, else 0
@@ -169,9 +169,10 @@ ACFX Num unpack(double x) {
     const uint64_t u = bits_of(x);
     const int hi = (int)(u >> 32);
     Num n;
+    const int ex = (hi >> 20) & 0x7ff;
     n.s = hi >> 31;
-    n.e = ((hi >> 20) & 0x7ff) - 1085;
-    n.m = ((u & 0xfffffffffffffull) | 0x10000000000000ull) << 10;
+    n.e = ex - 1085;
+    n.m = ex == 0 ? 0 : ((u & 0xfffffffffffffull) | 0x10000000000000ull) << 10;
     return n;
 }
 

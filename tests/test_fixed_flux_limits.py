@@ -115,3 +115,33 @@ def test_equal_pressures_or_velocities_hide_nothing(lib):
         assert check(lib, [rL, u, u * rng.normal(), p, rR, uR, u * rng.normal(), p], beta)
         dp = beta * 10 ** -rng.uniform(10, 40)
         assert check(lib, [rL, u, c * rng.normal(), dp, rR, u, c * rng.normal(), -dp], beta)
+
+
+@pytest.mark.parametrize("tiny", [0.0, -0.0, 5e-324, -5e-324, 1e-310, -2.2e-308])
+def test_signed_zeros_and_subnormals_beside_a_density_jump_and_a_pressure(lib, tiny):
+    """A velocity of zero of either sign, or subnormal, is a zero: at rest exactly the pressure, also where the sides'
+    densities differ; and a zero or subnormal pressure or tangential velocity gives what +0 gives."""
+    for rL, rR, p, v in ((1000.0, 1.0, 5.0, 0.3), (1.0, 1000.0, -7e3, -0.0), (2.0, 3.0, 1e-3, 1e3)):
+        for uL, uR in ((tiny, tiny), (tiny, 0.0), (0.0, tiny), (tiny, -tiny)):
+            assert flux(lib, [rL, uL, v, p, rR, uR, v, p], 4e5) == [0.0, 2.0 * p, 0.0, 0.0]
+        for q in (1, 2, 3, 5, 6, 7):
+            s = [rL, 0.2, 0.3, p, rR, -0.1, 0.4, 2 * p]
+            s[q] = 0.0
+            want = flux(lib, s, 4e5)
+            s[q] = tiny
+            assert flux(lib, s, 4e5) == want, (q, s)
+
+
+def test_the_sign_of_a_zero_changes_no_bit(lib):
+    """Random faces with some of u, v and p zero: +0, -0 and a subnormal give the same flux to the last bit."""
+    rng = np.random.default_rng(6)
+    for _ in range(4000):
+        s = (rng.uniform(-0.5, 0.5, 8) * 2.0 ** rng.uniform(-20, 20, 8))
+        s[[0, 4]] = np.abs(s[[0, 4]])
+        zero = [q for q in (1, 2, 3, 5, 6, 7) if rng.random() < 0.6]
+        beta = 2.0 ** rng.uniform(0, 20)
+        got = []
+        for tiny in (0.0, -0.0, -1e-310):
+            s[zero] = tiny
+            got.append(flux(lib, list(s), beta))
+        assert got[0] == got[1] == got[2], (list(s), beta)
