@@ -22,11 +22,13 @@ enum Riemann { kOsher = 0, kBassi = 1, kRoe = 2 };
 
 // ---------------------------------------------------------------------------
 // Arithmetic traits.  FP64 takes reciprocals and square roots on the integer
-// pipes (0.51 ulp; the FP64 unit spends 360-390 of its cycles per warp on the
-// library's, these take about 80 beside it), with the library's functions
-// where an argument or result is not a normal number; FP32 uses the fast
-// reciprocal / reciprocal-square-root instructions (about 1 ulp), which is far
-// below the FP32 rounding of the stored state.
+// pipes (the FP64 unit spends 360-390 of its cycles per warp on the library's,
+// these take about 80 beside it), correctly rounded like the library's, but to
+// 0.51 ulp as a pair of sqrt(x) and 1/sqrt(x) (rsqrt and a product: 1 ulp and
+// 1.5), with the library's functions where an argument or result is not a
+// normal number; FP32 uses the fast reciprocal / reciprocal-square-root
+// instructions (about 1 ulp), which is far below the FP32 rounding of the
+// stored state.
 // ---------------------------------------------------------------------------
 template <typename T> struct Ar;
 template <> struct Ar<double> {
@@ -41,10 +43,7 @@ template <> struct Ar<double> {
         }
     }
     static __device__ __forceinline__ double sqrt_(double x) {
-        double s = 0.0, rs;
-        if (!fx::rsqrt_ok(x)) return sqrt(x);
-        fx::sqrt_rsqrt(x, s, rs);
-        return s;
+        return fx::rsqrt_ok(x) ? fx::sqrt_rn(x) : sqrt(x);
     }
     static __device__ __forceinline__ double div(double a, double b) { return a / b; }
 };

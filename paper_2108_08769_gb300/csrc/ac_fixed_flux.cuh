@@ -274,28 +274,46 @@ ACFX uint64_t rsqrt61(uint64_t X) {
 }
 
 
-// 1/x to within 0.51 ulp, where x and 1/x are normal (rcp_ok).
+// 1/x correctly rounded, where x and 1/x are normal (rcp_ok): the quotient to within 0.51 units of 53 bits, then
+// one unit up or down where the remainder says so.
 ACFX bool rcp_ok(double x) { return ((uint32_t)(bits_of(x) >> 52) & 0x7ff) - 1u < 2044u; }
 ACFX double rcp(double x) {
     const uint64_t u = bits_of(x);
     const uint32_t hi = (uint32_t)(u >> 32);
-    const uint64_t m = ((u & 0xfffffffffffffull) | 0x10000000000000ull) << 9;
-    const uint64_t r = (rcp61(m) + 256) >> 9;            // [2^52, 2^53]
+    const uint64_t m = (u & 0xfffffffffffffull) | 0x10000000000000ull;   // [2^52, 2^53)
+    uint64_t r = (rcp61(m << 9) + 256) >> 9;             // 2^105/m, in [2^52, 2^53]
+    const int64_t e = -(int64_t)(r * m) * 2;             // 2 (2^105 - r m), from its low 64 bits; never a tie
+    r += (uint64_t)(e > (int64_t)m) - (uint64_t)(e < -(int64_t)m);
     const uint32_t ex = 2044u - ((hi >> 20) & 0x7ffu);
     return double_of(r + ((uint64_t)((ex << 20) | (hi & 0x80000000u)) << 32));
 }
-// sqrt(x) and 1/sqrt(x) to within 0.51 ulp, x positive and normal (rsqrt_ok).
+// Mantissa m 2^-62 in [1/4, 1) and half the (even) exponent of a positive normal x = m 2^(2h - 62) (rsqrt_ok).
+struct RootArg {
+    uint64_t m;
+    int h;
+};
 ACFX bool rsqrt_ok(double x) { return (uint32_t)(bits_of(x) >> 52) - 1u < 2046u; }
-ACFX void sqrt_rsqrt(double x, double &s, double &rs) {
+ACFX RootArg root_arg(double x) {
     const uint64_t u = bits_of(x);
     const int ex = (int)(u >> 52);
-    const int odd = ex & 1;                              // x = m 2^(ex - 1075); an even power of two either way
-    const uint64_t m = ((u & 0xfffffffffffffull) | 0x10000000000000ull) << (8 + (odd ^ 1));
-    const uint64_t y = rsqrt61(m);                       // x' = m 2^-62 in [1/4, 1), x = x' 2^(ex - 1021 - odd^1)
-    const int h = (ex - 1021 - (odd ^ 1)) / 2;           // exact: ex - 1021 - (odd ^ 1) is even
-    rs = double_of(((y + 256) >> 9) + ((uint64_t)(1022 - h) << 52));
-    const uint64_t c = mulu(m * 2, y * 2);               // sqrt(x') 2^61 in [2^60, 2^61]
-    s = double_of(((c + 128) >> 8) + ((uint64_t)(1021 + h) << 52));
+    const int even = (ex & 1) ^ 1;                       // an even power of two either way
+    return RootArg{((u & 0xfffffffffffffull) | 0x10000000000000ull) << (8 + even), (ex - 1021 - even) / 2};
+}
+// sqrt(x) and 1/sqrt(x) to within 0.51 ulp.
+ACFX void sqrt_rsqrt(double x, double &s, double &rs) {
+    const RootArg a = root_arg(x);
+    const uint64_t y = rsqrt61(a.m);
+    rs = double_of(((y + 256) >> 9) + ((uint64_t)(1022 - a.h) << 52));
+    const uint64_t c = mulu(a.m * 2, y * 2);             // sqrt(x') 2^61 in [2^60, 2^61]
+    s = double_of(((c + 128) >> 8) + ((uint64_t)(1021 + a.h) << 52));
+}
+// sqrt(x) correctly rounded, by its remainder as in rcp.
+ACFX double sqrt_rn(double x) {
+    const RootArg a = root_arg(x);
+    uint64_t s = (mulu(a.m * 2, rsqrt61(a.m) * 2) + 128) >> 8;           // sqrt(m 2^44), in [2^52, 2^53]
+    const int64_t e = (int64_t)((a.m << 44) - s * s);    // |e| < 1.1 s; (s +- 1/2)^2 is s^2 +- s and a quarter
+    s += (uint64_t)(e > (int64_t)s) - (uint64_t)(e <= -(int64_t)s);
+    return double_of(s + ((uint64_t)(1021 + a.h) << 52));
 }
 
 // |x|

@@ -145,3 +145,11 @@ def test_the_sign_of_a_zero_changes_no_bit(lib):
             s[zero] = tiny
             got.append(flux(lib, list(s), beta))
         assert got[0] == got[1] == got[2], (list(s), beta)
+
+
+@pytest.mark.parametrize("scale,scale_p", [(128.0, 51.2e6), (0.3, 7.7e-9), (1.0 / 3e5, 1e17), (1e-60, 1e60)])
+def test_factors_that_are_no_powers_of_two(lib, scale, scale_p):
+    rng = np.random.default_rng(11)
+    for ratio in (1e-6, 0.1, 3.0):
+        for s in draw(rng, ratio, 4e5, 10 ** rng.uniform(-3, 3)):
+            assert check(lib, s, 4e5, scale, scale_p)
