@@ -621,7 +621,7 @@ struct MixedBackend : Backend {
         a.beta = float(c->beta); a.inv_beta = float(1.0 / c->beta);
         a.gx = float(c->grid.gx); a.gy = float(c->grid.gy);
         a.cfl_area = float(c->opt.cfl_tau * dx * dy);
-        a.inv_cfl_area = float(1.0 / (c->opt.cfl_tau * dx * dy));
+        set_idt_scales(a, c->opt.cfl_tau, dx, dy);
         a.plevel = plevel ? 1 : 0;
         for (int b = 0; b < 3; ++b) a.d[b] = d[b];
         a.qn = qn;

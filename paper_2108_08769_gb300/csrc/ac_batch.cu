@@ -737,7 +737,7 @@ int ac_batch_create(int n, const ac_grid *grids, const double *beta, const ac_bc
         a.beta = float(beta[k]); a.inv_beta = float(1.0 / beta[k]);
         a.gx = float(g.gx); a.gy = float(g.gy);
         a.cfl_area = float(o.cfl_tau * dx * dy);
-        a.inv_cfl_area = float(1.0 / (o.cfl_tau * dx * dy));
+        set_idt_scales(a, o.cfl_tau, dx, dy);
         a.plevel = b->plevel ? 1 : 0;
         b->use_ref[k] = mixed_uses_reference(bcs[k], o.gradp);
         for (int x = 0; x < 3; ++x) a.d[x] = b->d[x] + pos;

@@ -57,7 +57,8 @@ struct MixedArgs {
     float dx, dy, half_dx, half_dy, inv_dx, inv_dy, dx_over_dy, dy_over_dx;
     float nh_inv_dx, nh_inv_dy;   // -1/(2 dx), -1/(2 dy)
     float beta, inv_beta, gx, gy;
-    float cfl_area, inv_cfl_area;
+    float cfl_area;
+    float idt_x, idt_y, idt_xl, idt_yl;   // 1/(2 CFL_tau dx), 1/(2 CFL_tau dy), each in two FP32 parts (set_idt_scales)
     int plevel;            // 1: pressure as dp over the FP64 level p^n; 0: the record holds p
     float4 *d[3];          // per cell (dQ of rho, rho u, rho v; dp or p), three rotating buffers
     float4 *qn;            // per cell (FP32 Q^n of rho, rho u, rho v; rho_ref)
@@ -74,6 +75,17 @@ struct MixedArgs {
     double *partials;
     Ctl *ctl;
 };
+
+// A cell's 1/dtau = (|u| + c_x)/(2 CFL_tau dx) + (|v| + c_y)/(2 CFL_tau dy).  One FP32 constant would put the same
+// relative error, up to 2^-24, on the pseudo-time step of every cell; the second parts take it away (p of a tank with
+// periodic sides after 60 iterations, rms: 4.4e-9 off 64 bits with one constant, 3.0e-9 without its error).
+inline void set_idt_scales(MixedArgs &a, double cfl_tau, double dx, double dy) {
+    const double x = 0.5 / (cfl_tau * dx), y = 0.5 / (cfl_tau * dy);
+    a.idt_x = float(x);
+    a.idt_y = float(y);
+    a.idt_xl = float(x - double(a.idt_x));
+    a.idt_yl = float(y - double(a.idt_y));
+}
 
 // Exact FP32 -> FP64 conversion with integer instructions (exponent rebias,
 // mantissa shift), off GB300's FP64 unit, which runs at 1/64 of the FP32
@@ -358,7 +370,8 @@ __device__ __forceinline__ void cell_update(const MixedArgs &a, float inv_alpha,
         const float u = m0 * ir, v = n0 * ir, fb = 4.0f * a.beta * ir;
         const float u2 = u * u + fb, v2 = v * v + fb;
         const float cx = u2 * rsqrtf(u2), cy = v2 * rsqrtf(v2);
-        idt = fmaf(fabsf(u) + cx, a.half_dy, (fabsf(v) + cy) * a.half_dx) * a.inv_cfl_area;
+        const float sx = fabsf(u) + cx, sy = fabsf(v) + cy;
+        idt = fmaf(sx, a.idt_x, fmaf(sy, a.idt_y, fmaf(sx, a.idt_xl, sy * a.idt_yl)));
         if constexpr (DTM == 1) {
             if (live) a.dtau[g] = idt;
         }
