@@ -18,11 +18,14 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <map>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -194,7 +197,29 @@ cudaError_t launch_f64(const SweepArgs<double> &a, dim3 g, bool pdl, cudaStream_
                       a);
 }
 
-std::vector<std::pair<std::pair<int, int>, int>> g_tuned_f64;
+// Variants that the autotuners chose, shared by the contexts of this process:
+// per form (its own cache), device, grid and the options that decide which
+// instance or path a stage runs.
+struct TuneCache {
+    using Key = std::array<int, 10>;
+    std::mutex m;
+    std::map<Key, int> chosen;
+    static Key key(const ac_ctx *c) {
+        const ac_options &o = c->opt;
+        return Key{c->device, c->grid.nx, c->grid.ny, o.rk_stages, o.gradp, o.limiter_k,
+                   o.local_dtau, o.realtime, o.alpha_pi_p_row, o.bdf_order};
+    }
+    int find(const ac_ctx *c) {   // -1: not tuned yet
+        const std::lock_guard<std::mutex> lock(m);
+        const auto it = chosen.find(key(c));
+        return it == chosen.end() ? -1 : it->second;
+    }
+    void put(const ac_ctx *c, int v) {
+        const std::lock_guard<std::mutex> lock(m);
+        chosen[key(c)] = v;
+    }
+};
+TuneCache g_tuned_f64, g_tuned;
 
 struct F64Backend : Backend {
     int variant = -1;
@@ -243,7 +268,7 @@ struct F64Backend : Backend {
 
     // Autotuner: one pseudo-iteration's stages of every shape on this grid
     // (they write only the two scratch buffers and the residual partials,
-    // all rewritten by the real iteration), fastest kept per grid size.
+    // all rewritten by the real iteration), fastest kept (TuneCache).
     int tune(ac_ctx *c, cudaStream_t s) override {
         if (variant >= 0) return AC_OK;
         if (c->opt.riemann != AC_RIEMANN_OSHER) { set_variant(c, 0); return AC_OK; }
@@ -252,13 +277,16 @@ struct F64Backend : Backend {
             const int v = atoi(env);
             if (v >= 0 && v < kNumF64Variants) { set_variant(c, v); return AC_OK; }
         }
-        for (auto &kv : g_tuned_f64)
-            if (kv.first.first == c->grid.nx && kv.first.second == c->grid.ny) {
-                set_variant(c, kv.second);
-                return AC_OK;
-            }
-        // the scratch buffers start as copies of the state, so that every
-        // timed stage sees real data
+        if (const int v = g_tuned_f64.find(c); v >= 0) { set_variant(c, v); return AC_OK; }
+        // with the global pseudo-time step, the step that the first iteration
+        // will find again (a step's beginning leaves it at +inf, and stages
+        // timed past it would run on states without meaning); the scratch
+        // buffers start as copies of the state
+        if (!c->opt.local_dtau) {
+            const int rc = dtau_min(c, s);
+            if (rc != AC_OK) return rc;
+            c->launches += 1;
+        }
         for (int b = 0; b < 3; ++b)
             if (b != c->cur_host)
                 for (int f = 0; f < 4; ++f)
@@ -289,7 +317,7 @@ struct F64Backend : Backend {
             }
         const int best = int(std::min_element(tmin.begin(), tmin.end()) - tmin.begin());
         set_variant(c, best);
-        g_tuned_f64.push_back({{c->grid.nx, c->grid.ny}, best});
+        g_tuned_f64.put(c, best);
         return AC_OK;
     }
 
@@ -474,12 +502,6 @@ cudaError_t allow_mixed_smem() {
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(MixedSmem<TX, TY>));
 }
 
-// chosen tile shape per grid size, shared by the contexts of this process
-struct TuneKey {
-    int nx, ny;
-};
-std::vector<std::pair<TuneKey, int>> g_tuned;
-
 struct MixedBackend : Backend {
     int variant = -1;
     float4 *d[3] = {};   // per cell (dQ of rho, rho u, rho v; dp or p), three rotating buffers
@@ -562,13 +584,16 @@ struct MixedBackend : Backend {
                 return AC_OK;
             }
         }
-        for (auto &kv : g_tuned)
-            if (kv.first.nx == c->grid.nx && kv.first.ny == c->grid.ny && (sweep_ok || !kMixedVariants[kv.second].sweep)) {
-                set_variant(c, kv.second);
-                return AC_OK;
-            }
-        // the scratch buffers start as copies of the state, so that every
-        // timed stage sees real data
+        if (const int v = g_tuned.find(c); v >= 0) { set_variant(c, v); return AC_OK; }
+        // with the global pseudo-time step, the step that the first iteration
+        // will find again (a step's beginning leaves it at +inf, and stages
+        // timed past it would run on states without meaning); the scratch
+        // buffers start as copies of the state
+        if (!c->opt.local_dtau) {
+            const int rc = dtau_min(c, s);
+            if (rc != AC_OK) return rc;
+            c->launches += 1;
+        }
         for (int b = 0; b < 3; ++b)
             if (b != c->cur_host)
                 CK(cudaMemcpyAsync(d[b], d[c->cur_host], c->N * sizeof(float4), cudaMemcpyDeviceToDevice, s));
@@ -599,7 +624,7 @@ struct MixedBackend : Backend {
             }
         const int best = int(std::min_element(tmin.begin(), tmin.end()) - tmin.begin());
         set_variant(c, best);
-        g_tuned.push_back({TuneKey{c->grid.nx, c->grid.ny}, best});
+        g_tuned.put(c, best);
         return AC_OK;
     }
 
