@@ -86,6 +86,13 @@ constexpr int kGridStrideBlocks = 152 * 8;
 
 bool valid_bc(int b) { return b >= AC_BC_WALL_SLIP && b <= AC_BC_PERIODIC; }
 
+// A captured physical step and the backward-difference order it was built for.
+struct StepGraph {
+    cudaGraph_t graph;
+    cudaGraphExec_t exec;
+    int order;
+};
+
 struct Backend;
 
 }  // namespace
@@ -106,8 +113,7 @@ struct ac_ctx {
     Ctl *hctl;            // pinned host mirror
     cudaStream_t stream;  // user stream (0 = default)
     cudaStream_t cap;     // private stream used for capture
-    cudaGraph_t graph;
-    cudaGraphExec_t exec;
+    StepGraph steps[2];   // the captured step, and for steps that may end at once (see may_end_at_once)
     bool has_state;
     int cur_host;
     long long launches;
@@ -120,7 +126,6 @@ struct ac_ctx {
     bool pdl;             // launch the loop's kernels with programmatic dependencies
     int nhist;            // older real-time levels held (0..2) before the next step
     int order_now;        // backward-difference order of the current step
-    int graph_order;      // order the captured graph was built for
 };
 
 namespace {
@@ -882,28 +887,30 @@ int kernels_per_iteration(const ac_ctx *c) {
     return c->opt.rk_stages + 1 + (c->opt.local_dtau ? 0 : 1) + c->be->kernels_after_iteration();
 }
 
-int build_graph(ac_ctx *c) {
-    if (c->exec && c->graph_order == c->order_now) return AC_OK;
-    if (c->exec) {
-        cudaGraphExecDestroy(c->exec);
-        cudaGraphDestroy(c->graph);
-        c->exec = nullptr;
-        c->graph = nullptr;
-    }
-    c->graph_order = c->order_now;
-    CK(cudaGraphCreate(&c->graph, 0));
+// Iterations in line ahead of a captured step's loop: with a pressure rebase
+// those up to the last one, else two where the step may end right after them.
+int lead_iters(const ac_ctx *c, bool at_once) { return c->be->rebases() ? kRebaseLast : at_once ? kAtOnceIters : 0; }
+
+int build_graph(ac_ctx *c, bool at_once) {
+    StepGraph &sg = c->steps[at_once];
+    if (sg.exec && sg.order == c->order_now) return AC_OK;
+    if (sg.exec) cudaGraphExecDestroy(sg.exec);
+    if (sg.graph) cudaGraphDestroy(sg.graph);
+    sg = StepGraph{nullptr, nullptr, c->order_now};
+    CK(cudaGraphCreate(&sg.graph, 0));
     cudaGraphConditionalHandle h;
-    CK(cudaGraphConditionalHandleCreate(&h, c->graph, 1, cudaGraphCondAssignDefault));
-    // With a pressure rebase (mixed form) the first kRebaseLast pseudo-iterations
-    // run in line ahead of the loop, the rebase kernels after iterations 1, 2,
-    // 4, 8 only, so that the loop body itself carries no per-iteration node
-    // for them.  Each of these iterations sets the loop's condition; once
-    // the step is done their kernels return at once.
+    CK(cudaGraphConditionalHandleCreate(&h, sg.graph, 1, cudaGraphCondAssignDefault));
+    // The first pseudo-iterations run in line ahead of the loop (lead_iters).
+    // With a pressure rebase (mixed form) the rebase kernels follow iterations
+    // 1, 2, 4, 8 only, so that the loop body itself carries no per-iteration
+    // node for them.  Each of these iterations sets the loop's condition;
+    // once the step is done their kernels return at once.
+    const int lead = lead_iters(c, at_once);
     std::vector<cudaGraphNode_t> pro;
-    if (c->be->rebases()) {
-        CK(cudaStreamBeginCaptureToGraph(c->cap, c->graph, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
+    if (lead > 0) {
+        CK(cudaStreamBeginCaptureToGraph(c->cap, sg.graph, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
         int rc = AC_OK;
-        for (int m = 1; m <= kRebaseLast && rc == AC_OK; ++m)
+        for (int m = 1; m <= lead && rc == AC_OK; ++m)
             rc = enqueue_iteration(c, c->cap, (unsigned long long)h, 1, false, rebase_after(m));
         cudaStreamCaptureStatus st;
         cudaGraph_t g = nullptr;
@@ -926,7 +933,7 @@ int build_graph(ac_ctx *c) {
     cp.conditional.type = cudaGraphCondTypeWhile;
     cp.conditional.size = 1;
     cudaGraphNode_t node;
-    CK(cudaGraphAddNode(&node, c->graph, pro.empty() ? nullptr : pro.data(), nullptr, pro.size(), &cp));
+    CK(cudaGraphAddNode(&node, sg.graph, pro.empty() ? nullptr : pro.data(), nullptr, pro.size(), &cp));
     cudaGraph_t body = cp.conditional.phGraph_out[0];
     CK(cudaStreamBeginCaptureToGraph(c->cap, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
     int rc = AC_OK;
@@ -936,7 +943,7 @@ int build_graph(ac_ctx *c) {
     cudaError_t e = cudaStreamEndCapture(c->cap, &captured);
     if (rc != AC_OK) return rc;
     if (e != cudaSuccess) return fail(AC_ERR_CUDA, "graph capture failed: %s", cudaGetErrorString(e));
-    CK(cudaGraphInstantiate(&c->exec, c->graph, 0));
+    CK(cudaGraphInstantiate(&sg.exec, sg.graph, 0));
     return AC_OK;
 }
 
@@ -1062,8 +1069,10 @@ void ac_destroy(ac_ctx *c) {
     if (c->stream) cudaStreamSynchronize(c->stream);
     for (int k = 0; k < 5; ++k)
         if (c->ev[k]) cudaEventDestroy(c->ev[k]);
-    if (c->exec) cudaGraphExecDestroy(c->exec);
-    if (c->graph) cudaGraphDestroy(c->graph);
+    for (StepGraph &g : c->steps) {
+        if (g.exec) cudaGraphExecDestroy(g.exec);
+        if (g.graph) cudaGraphDestroy(g.graph);
+    }
     if (c->cap) cudaStreamDestroy(c->cap);
     if (c->be) { c->be->release(); delete c->be; }
     cudaFree(c->partials);
@@ -1176,19 +1185,18 @@ static int physical_step_impl(ac_ctx *c, double dt, double tol, int max_iters, i
         }
         c->launches += (long long)launched * kernels_per_iteration(c);
     } else {
-        if ((rc = build_graph(c)) != AC_OK) return rc;
-        CK(cudaGraphLaunch(c->exec, s));
+        // without a rebase, which always has iterations in line, and for a step in real time
+        const bool at_once = !c->be->rebases() && !(tau_end < INFINITY) && may_end_at_once(tol, max_iters);
+        if ((rc = build_graph(c, at_once)) != AC_OK) return rc;
+        CK(cudaGraphLaunch(c->steps[at_once].exec, s));
         CK(cudaMemcpyAsync(c->hctl, c->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
-        // with a rebase the graph's in-line prologue always launches its
-        // kRebaseLast iterations and four rebase pairs (returning at once
-        // once the step is done); the loop runs the rest
+        // the iterations in line are always launched, with a rebase their four
+        // rebase pairs too (returning at once once the step is done); the loop
+        // runs the rest
         const int ka = c->be->kernels_after_iteration();
-        if (c->be->rebases())
-            c->launches += launched_iters(c->hctl->iter, kRebaseLast) * (kernels_per_iteration(c) - ka) +
-                           rebases_in(kRebaseLast + 1) * ka;
-        else
-            c->launches += launched_iters(c->hctl->iter, 0) * kernels_per_iteration(c);
+        c->launches += launched_iters(c->hctl->iter, lead_iters(c, at_once)) * (kernels_per_iteration(c) - ka) +
+                       (c->be->rebases() ? rebases_in(kRebaseLast + 1) * ka : 0);
     }
     if (iters_out) *iters_out = c->hctl->iter;
     if (c->hctl->status == -3) {

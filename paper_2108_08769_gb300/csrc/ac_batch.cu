@@ -50,6 +50,12 @@ struct BatchTank {
     int pad;
 };
 
+// Conditions of a captured step that the end of an iteration sets to whether any tank goes on.
+struct BatchEnd {
+    int n;
+    unsigned long long cond[2];
+};
+
 struct BatchSync {
     unsigned int arrive;       // end-of-iteration CTAs arrived
     unsigned int still_active; // tanks still iterating after this iteration
@@ -192,7 +198,7 @@ __global__ void batch_rebase_jumps_kernel(const BatchTank *tanks) {
 // CTA sets the WHILE condition.
 template <int NT>
 __global__ void __launch_bounds__(NT)
-batch_end_kernel(BatchTank *tanks, BatchSync *sync, int ntanks, unsigned long long cond, int use_cond) {
+batch_end_kernel(BatchTank *tanks, BatchSync *sync, int ntanks, const BatchEnd end) {
     static_assert(NT >= kEndLanes, "sum_partials_fixed needs kEndLanes threads");
     const int tid = threadIdx.x;
     pdl_wait();
@@ -228,7 +234,7 @@ batch_end_kernel(BatchTank *tanks, BatchSync *sync, int ntanks, unsigned long lo
             __threadfence();
             const unsigned int left = atomicExch(&sync->still_active, 0u);
             sync->arrive = 0;
-            if (use_cond) cudaGraphSetConditional(cond, left ? 1u : 0u);
+            for (int k = 0; k < end.n; ++k) cudaGraphSetConditional(end.cond[k], left ? 1u : 0u);
         }
     }
 }
@@ -365,8 +371,8 @@ struct ac_batch {
     int ntiles;
     std::vector<int> map_host;
     cudaStream_t stream, cap;
-    cudaGraph_t graph;
-    cudaGraphExec_t exec;
+    cudaGraph_t graph[2];               // the captured step, and for steps that may end at once (see build_graph)
+    cudaGraphExec_t exec[2];
     bool has_state;
     int nhist;                          // older real-time levels held before the next step
     int order_now;                      // backward-difference order in the descriptors
@@ -507,15 +513,14 @@ int tune(ac_batch *b, cudaStream_t s) {
 }
 
 // One pseudo-iteration; rebase adds the kernels that act after iterations 1, 2, 4, 8.
-int enqueue_iteration(ac_batch *b, cudaStream_t s, unsigned long long cond, int use_cond, bool timed, bool rebase) {
+int enqueue_iteration(ac_batch *b, cudaStream_t s, const BatchEnd &end, bool timed, bool rebase) {
     int rc;
     if (timed) CK(cudaEventRecord(b->ev[0], s));
     for (int st = 1; st <= b->opt.rk_stages; ++st) {
         if ((rc = stage_launch(b, s, st, b->variant)) != AC_OK) return rc;
         if (timed) CK(cudaEventRecord(b->ev[st], s));
     }
-    CK(launch_pdl(b->pdl, batch_end_kernel<256>, dim3(b->n), dim3(256), 0, s, b->tanks_dev, b->sync, b->n, cond,
-                  use_cond));
+    CK(launch_pdl(b->pdl, batch_end_kernel<256>, dim3(b->n), dim3(256), 0, s, b->tanks_dev, b->sync, b->n, end));
     CK(cudaGetLastError());
     if (b->plevel && rebase) {
         CK(launch_pdl(b->pdl, batch_rebase_shift_kernel, b->rebase_grid, dim3(256), 0, s, b->tanks_dev));
@@ -524,50 +529,77 @@ int enqueue_iteration(ac_batch *b, cudaStream_t s, unsigned long long cond, int 
     return AC_OK;
 }
 
-// As the single tank's graph: with a pressure rebase the first kRebaseLast
-// iterations run in line ahead of the loop, the rebase kernels only where
-// they act (every tank still iterating is at the same iteration), and the
-// loop's body holds kLoopIters iterations without them.
-int build_graph(ac_batch *b) {
-    if (b->exec) return AC_OK;
-    CK(cudaGraphCreate(&b->graph, 0));
-    cudaGraphConditionalHandle h;
-    CK(cudaGraphConditionalHandleCreate(&h, b->graph, 1, cudaGraphCondAssignDefault));
-    std::vector<cudaGraphNode_t> pro;
+// Iterations first .. last captured into g after deps (which receives their last nodes), the rebase kernels only where
+// they act (every tank still iterating is at the same iteration).
+int capture_iterations(ac_batch *b, cudaGraph_t g, std::vector<cudaGraphNode_t> *deps, const BatchEnd &end, int first,
+                       int last) {
+    CK(cudaStreamBeginCaptureToGraph(b->cap, g, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
     int rc = AC_OK;
-    if (b->plevel) {
-        CK(cudaStreamBeginCaptureToGraph(b->cap, b->graph, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-        for (int m = 1; m <= kRebaseLast && rc == AC_OK; ++m)
-            rc = enqueue_iteration(b, b->cap, (unsigned long long)h, 1, false, rebase_after(m));
-        cudaStreamCaptureStatus st;
-        cudaGraph_t g = nullptr, captured = nullptr;
-        const cudaGraphNode_t *deps = nullptr;
-        size_t nd = 0;
-        cudaError_t e = cudaStreamGetCaptureInfo(b->cap, &st, nullptr, &g, &deps, nullptr, &nd);
-        if (e == cudaSuccess) pro.assign(deps, deps + nd);
-        const cudaError_t e2 = cudaStreamEndCapture(b->cap, &captured);
-        if (rc != AC_OK) return rc;
-        if (e != cudaSuccess || e2 != cudaSuccess)
-            return fail(AC_ERR_CUDA, "graph capture failed: %s", cudaGetErrorString(e != cudaSuccess ? e : e2));
-    }
+    for (int m = first; m <= last && rc == AC_OK; ++m) rc = enqueue_iteration(b, b->cap, end, false, rebase_after(m));
+    cudaStreamCaptureStatus st;
+    cudaGraph_t captured = nullptr;
+    const cudaGraphNode_t *nodes = nullptr;
+    size_t nd = 0;
+    const cudaError_t e = cudaStreamGetCaptureInfo(b->cap, &st, nullptr, &captured, &nodes, nullptr, &nd);
+    if (deps && e == cudaSuccess) deps->assign(nodes, nodes + nd);
+    const cudaError_t e2 = cudaStreamEndCapture(b->cap, &captured);
+    if (rc != AC_OK) return rc;
+    if (e != cudaSuccess || e2 != cudaSuccess)
+        return fail(AC_ERR_CUDA, "graph capture failed: %s", cudaGetErrorString(e != cudaSuccess ? e : e2));
+    return AC_OK;
+}
+
+// A conditional node after deps (which receives it): iterations first .. last once or in a loop.
+int add_conditional(ac_batch *b, cudaGraph_t g, std::vector<cudaGraphNode_t> &deps, cudaGraphConditionalHandle h,
+                    cudaGraphConditionalNodeType type, const BatchEnd &end, int first, int last) {
     alignas(cudaGraphNodeParams) unsigned char cp_raw[sizeof(cudaGraphNodeParams)];
     memset(cp_raw, 0, sizeof cp_raw);
     cudaGraphNodeParams &cp = *reinterpret_cast<cudaGraphNodeParams *>(cp_raw);
     cp.type = cudaGraphNodeTypeConditional;
     cp.conditional.handle = h;
-    cp.conditional.type = cudaGraphCondTypeWhile;
+    cp.conditional.type = type;
     cp.conditional.size = 1;
     cudaGraphNode_t node;
-    CK(cudaGraphAddNode(&node, b->graph, pro.empty() ? nullptr : pro.data(), nullptr, pro.size(), &cp));
-    cudaGraph_t body = cp.conditional.phGraph_out[0];
-    CK(cudaStreamBeginCaptureToGraph(b->cap, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-    for (int m = 0; m < kLoopIters && rc == AC_OK; ++m)
-        rc = enqueue_iteration(b, b->cap, (unsigned long long)h, 1, false, false);
-    cudaGraph_t captured = nullptr;
-    const cudaError_t e = cudaStreamEndCapture(b->cap, &captured);
-    if (rc != AC_OK) return rc;
-    if (e != cudaSuccess) return fail(AC_ERR_CUDA, "graph capture failed: %s", cudaGetErrorString(e));
-    CK(cudaGraphInstantiate(&b->exec, b->graph, 0));
+    CK(cudaGraphAddNode(&node, g, deps.empty() ? nullptr : deps.data(), nullptr, deps.size(), &cp));
+    deps.assign(1, node);
+    return capture_iterations(b, cp.conditional.phGraph_out[0], nullptr, end, first, last);
+}
+
+// Iterations that a captured step always runs in line, and all that it runs
+// ahead of its loop: with a pressure rebase the first kRebaseLast, else none.
+// A step that may end at once (may_end_at_once) runs two in line and the
+// others, if any, as the body of an IF (six tanks of 20 to 40 cells a side,
+// steps that end after 1 and 2 iterations: 117 and 140 us with eight in line,
+// 89 and 110; entering the IF takes about 10).
+int lead_iters(const ac_batch *b, bool at_once) { return at_once ? kAtOnceIters : b->plevel ? kRebaseLast : 0; }
+int before_loop(const ac_batch *b, bool at_once) { return b->plevel ? kRebaseLast : at_once ? kAtOnceIters : 0; }
+
+// The captured step; the loop's body holds kLoopIters iterations without rebase kernels.
+int build_graph(ac_batch *b, bool at_once) {
+    if (b->exec[at_once]) return AC_OK;
+    cudaGraph_t &g = b->graph[at_once];
+    if (g) cudaGraphDestroy(g);
+    g = nullptr;
+    CK(cudaGraphCreate(&g, 0));
+    const int lead = lead_iters(b, at_once), before = before_loop(b, at_once);
+    cudaGraphConditionalHandle loop, rest = 0;
+    CK(cudaGraphConditionalHandleCreate(&loop, g, 1, cudaGraphCondAssignDefault));
+    BatchEnd end{1, {(unsigned long long)loop, 0}};
+    std::vector<cudaGraphNode_t> deps;
+    int rc = AC_OK;
+    if (lead < before) {
+        CK(cudaGraphConditionalHandleCreate(&rest, g, 1, cudaGraphCondAssignDefault));
+        end = BatchEnd{2, {(unsigned long long)loop, (unsigned long long)rest}};
+    }
+    if (lead > 0 && (rc = capture_iterations(b, g, &deps, end, 1, lead)) != AC_OK) return rc;
+    end.n = 1;
+    if (lead < before && (rc = add_conditional(b, g, deps, rest, cudaGraphCondTypeIf, end, lead + 1, before)) != AC_OK)
+        return rc;
+    // (past the rebases' iterations)
+    if ((rc = add_conditional(b, g, deps, loop, cudaGraphCondTypeWhile, end, kRebaseLast + 1,
+                              kRebaseLast + kLoopIters)) != AC_OK)
+        return rc;
+    CK(cudaGraphInstantiate(&b->exec[at_once], g, 0));
     return AC_OK;
 }
 
@@ -589,8 +621,10 @@ void ac_batch_destroy(ac_batch *b) {
     cudaStreamSynchronize(b->stream);   // (0: the default stream) nothing of this batch still runs
     for (int k = 0; k < 5; ++k)
         if (b->ev[k]) cudaEventDestroy(b->ev[k]);
-    if (b->exec) cudaGraphExecDestroy(b->exec);
-    if (b->graph) cudaGraphDestroy(b->graph);
+    for (int g = 0; g < 2; ++g) {
+        if (b->exec[g]) cudaGraphExecDestroy(b->exec[g]);
+        if (b->graph[g]) cudaGraphDestroy(b->graph[g]);
+    }
     if (b->cap) cudaStreamDestroy(b->cap);
     for (int x = 0; x < 3; ++x) cudaFree(b->d[x]);
     cudaFree(b->qn);
@@ -882,10 +916,9 @@ static int batch_step_impl(ac_batch *b, const double *dt, double tol, int max_it
     int rc = tune(b, s);
     if (rc != AC_OK) return rc;
     b->pdl = pdl_enabled() && !b->profiling;
-    long long iters_run = 0;
     if (b->profiling) {
         while (true) {
-            if ((rc = enqueue_iteration(b, s, 0, 0, true, true)) != AC_OK) return rc;
+            if ((rc = enqueue_iteration(b, s, BatchEnd{}, true, true)) != AC_OK) return rc;
             CK(cudaMemcpyAsync(b->hctl, b->ctl, b->n * sizeof(Ctl), cudaMemcpyDeviceToHost, s));
             CK(cudaStreamSynchronize(s));
             for (int st = 1; st <= b->opt.rk_stages; ++st) {
@@ -894,23 +927,27 @@ static int batch_step_impl(ac_batch *b, const double *dt, double tol, int max_it
                 b->stage_ms += ms;
             }
             b->stage_launches += b->opt.rk_stages;
-            ++iters_run;
+            b->launches += b->opt.rk_stages + 1 + (b->plevel ? 2 : 0);
             bool all = true;
             for (int k = 0; k < b->n; ++k) all = all && b->hctl[k].done;
             if (all) break;
         }
     } else {
-        if ((rc = build_graph(b)) != AC_OK) return rc;
-        CK(cudaGraphLaunch(b->exec, s));
+        const bool at_once = may_end_at_once(tol, max_iters);
+        if ((rc = build_graph(b, at_once)) != AC_OK) return rc;
+        CK(cudaGraphLaunch(b->exec[at_once], s));
         CK(cudaMemcpyAsync(b->hctl, b->ctl, b->n * sizeof(Ctl), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
-        for (int k = 0; k < b->n; ++k) iters_run = std::max<long long>(iters_run, b->hctl[k].iter);
+        int it = 0;
+        for (int k = 0; k < b->n; ++k) it = std::max(it, b->hctl[k].iter);
+        // the iterations in line with their rebase pairs, those under the IF
+        // with theirs where it ran, then whole bodies of the loop
+        const int lead = lead_iters(b, at_once), before = before_loop(b, at_once);
+        const int line = it > lead ? before : lead;
+        int pairs = 0;
+        for (int m = 1; m <= line && b->plevel; ++m) pairs += rebase_after(m);
+        b->launches += launched_iters(it, line) * (b->opt.rk_stages + 1) + 2 * pairs;
     }
-    if (b->profiling)
-        b->launches += iters_run * (b->opt.rk_stages + 1 + (b->plevel ? 2 : 0));
-    else   // the in-line iterations with their four rebase pairs, then whole bodies of the loop
-        b->launches += launched_iters(iters_run, b->plevel ? kRebaseLast : 0) * (b->opt.rk_stages + 1) +
-                       (b->plevel ? 8 : 0);
     int ret = AC_OK;
     bool any_nonfinite = false;
     for (int k = 0; k < b->n; ++k) {

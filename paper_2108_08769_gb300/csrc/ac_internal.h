@@ -28,11 +28,22 @@ inline bool pdl_enabled() {
 }
 
 // Pseudo-iterations in a captured loop's body: evaluating the loop's condition
-// costs 2-3 us, a tenth of a small grid's iteration (with the first stage
-// launched plainly: 20x20 mixed 22.9 -> 20.7 us, FP64 57.7 -> 55.8, 256x256
-// mixed 28.9 -> 27.0; eight gain 1 us more).  Iterations past the step's end
-// return at once.
+// costs 3 us, a tenth of a small grid's iteration (FP64 20x20, steps of 17 and
+// 33: 745 and 1421 us with one iteration to a body, 723 and 1366 with four).
+// Iterations past the step's end return at once, which takes 4 us an iteration
+// on small grids and 8 on 1024x512: a step that ends after one or two loses by
+// the body of four (70 and 108 us with one to a body, 81 and 118 with four),
+// from the third on it gains or is even.
 constexpr int kLoopIters = 4;
+
+// A step that may well end after one or two pseudo-iterations, as its number
+// of them says or because it stops on its tolerance (a tank that has come to
+// rest starts every step below it), runs two in line ahead of its loop: 71 and
+// 108 us on that grid.  Longer steps that stop on a tolerance then gain or
+// lose by where they end in a body (100x1, 3 to 6 iterations: 132, 166, 208,
+// 242 -> 143, 172, 204, 231; 33: 1154 -> 1163); fixed numbers keep the loop alone.
+constexpr int kAtOnceIters = 2;
+inline bool may_end_at_once(double tol, int max_iters) { return tol >= 0.0 || max_iters <= kAtOnceIters; }
 
 // Iterations whose kernels a step of `iters` launches: `lead` in line, then whole bodies of the loop.
 inline long long launched_iters(long long iters, int lead) {
