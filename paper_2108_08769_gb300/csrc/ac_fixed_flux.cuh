@@ -159,8 +159,9 @@ ACFX uint64_t bits_of(double x) {
 #endif
 }
 
-// A double as sign, 63-bit mantissa in [2^62, 2^63) and exponent.  Zeros and subnormals have no mantissa: a number
-// near 2^-1022 instead would leave -1 behind where a negative one is shifted far to the right.
+// A double as sign, 63-bit mantissa in [2^62, 2^63) and exponent.  Zeros and subnormals become positive numbers near
+// 2^-1022, which vanish beside any normal number (a negative one would leave -1 behind where it is shifted far to the
+// right) and which to_double makes zero again.
 struct Num {
     uint64_t m;
     int e, s;   // s = -1 for a negative number, else 0
@@ -170,9 +171,9 @@ ACFX Num unpack(double x) {
     const int hi = (int)(u >> 32);
     Num n;
     const int ex = (hi >> 20) & 0x7ff;
-    n.s = hi >> 31;
+    n.s = ex == 0 ? 0 : hi >> 31;
     n.e = ex - 1085;
-    n.m = ex == 0 ? 0 : ((u & 0xfffffffffffffull) | 0x10000000000000ull) << 10;
+    n.m = ((u & 0xfffffffffffffull) | 0x10000000000000ull) << 10;
     return n;
 }
 
@@ -274,16 +275,16 @@ ACFX uint64_t rsqrt61(uint64_t X) {
 }
 
 
-// 1/x correctly rounded, where x and 1/x are normal (rcp_ok): the quotient to within 0.51 units of 53 bits, then
-// one unit up or down where the remainder says so.
+// 1/x correctly rounded, where x and 1/x are normal (rcp_ok): the quotient's rounding or one unit less, by a limit
+// 8 units of 2^61 (the iteration's error) above the half, then one unit up where the remainder says so.
 ACFX bool rcp_ok(double x) { return ((uint32_t)(bits_of(x) >> 52) & 0x7ff) - 1u < 2044u; }
 ACFX double rcp(double x) {
     const uint64_t u = bits_of(x);
     const uint32_t hi = (uint32_t)(u >> 32);
     const uint64_t m = (u & 0xfffffffffffffull) | 0x10000000000000ull;   // [2^52, 2^53)
-    uint64_t r = (rcp61(m << 9) + 256) >> 9;             // 2^105/m, in [2^52, 2^53]
+    uint64_t r = (rcp61(m << 9) + 248) >> 9;             // 2^105/m, in [2^52, 2^53], or one less
     const int64_t e = -(int64_t)(r * m) * 2;             // 2 (2^105 - r m), from its low 64 bits; never a tie
-    r += (uint64_t)(e > (int64_t)m) - (uint64_t)(e < -(int64_t)m);
+    r += e > (int64_t)m;
     const uint32_t ex = 2044u - ((hi >> 20) & 0x7ffu);
     return double_of(r + ((uint64_t)((ex << 20) | (hi & 0x80000000u)) << 32));
 }
@@ -310,9 +311,9 @@ ACFX void sqrt_rsqrt(double x, double &s, double &rs) {
 // sqrt(x) correctly rounded, by its remainder as in rcp.
 ACFX double sqrt_rn(double x) {
     const RootArg a = root_arg(x);
-    uint64_t s = (mulu(a.m * 2, rsqrt61(a.m) * 2) + 128) >> 8;           // sqrt(m 2^44), in [2^52, 2^53]
-    const int64_t e = (int64_t)((a.m << 44) - s * s);    // |e| < 1.1 s; (s +- 1/2)^2 is s^2 +- s and a quarter
-    s += (uint64_t)(e > (int64_t)s) - (uint64_t)(e <= -(int64_t)s);
+    uint64_t s = (mulu(a.m * 2, rsqrt61(a.m) * 2) + 112) >> 8;           // sqrt(m 2^44), in [2^52, 2^53], or one less
+    const int64_t e = (int64_t)((a.m << 44) - s * s);    // below 3.1 s; (s + 1/2)^2 is s^2 + s and a quarter
+    s += e > (int64_t)s;
     return double_of(s + ((uint64_t)(1021 + a.h) << 52));
 }
 
@@ -381,16 +382,17 @@ ACFX void osher_flux_fixed(double rLd, double uLd, double vLd, double pLd, doubl
     // jumps of p and u as signs and magnitudes in [2^61, 2^62); the point sums below are formed times sd = sign(du)
     const int sd = (int)(DU >> 63), sp = (int)(DPs >> 63) ^ sd;
     uint64_t DP = mag(DPs), du = mag(DU);
-    // a zero jump's exponent is below all others, so that no common exponent is formed for its sake
-    const int none = -16384;
-    const int kd = room(DP), ku = room(du), epd = DP == 0 ? none : ep - kd;
+    const int kd = room(DP), ku = room(du);
     DP <<= kd;
     du <<= ku;
+    // a zero jump's exponent is below all others, so that no common exponent is formed for its sake
+    const int none = -16384;
+    const int epd = (uint32_t)(DP >> 32) == 0 ? none : ep - kd;
     // 2 rho_L rho_R |du| in [2^62, 2^63) (or 0)
     uint64_t D = mulu(mulu(rL.m, rR.m) * 2, du * 2);     // [2^59, 2^62)
     const int kD = clz32((uint32_t)(D >> 32) | 1u) - 1;
     D <<= kD;
-    int eb = du == 0 ? none : rL.e + rR.e + (ed - ku) + 128 - kD - er;
+    int eb = (uint32_t)(du >> 32) == 0 ? none : rL.e + rR.e + (ed - ku) + 128 - kD - er;
     // ---- first loop: u, c, a, b at the Gauss points (twice the states: r' = rS -+ t dr, m' = c0 -+ t dm) ----
     const int64_t TR = neg_if((int64_t)mulhi(kT64, mag(DR)), (int)(DR >> 63));
     const int64_t TM = neg_if((int64_t)mulhi(kT64, mag(DM)), (int)(DM >> 63));
