@@ -82,7 +82,6 @@ size_t max_tiles(int nx, int ny) {
         m = std::max(m, (size_t)((nx + sh[0] - 1) / sh[0]) * ((ny + sh[1] - 1) / sh[1]));
     return m;
 }
-constexpr int kGridStrideBlocks = 152 * 8;
 
 bool valid_bc(int b) { return b >= AC_BC_WALL_SLIP && b <= AC_BC_PERIODIC; }
 
@@ -129,8 +128,6 @@ struct ac_ctx {
 };
 
 namespace {
-
-int grid_stride_blocks(size_t N) { return (int)std::min<size_t>((N + 255) / 256, kGridStrideBlocks); }
 
 struct Backend {
     dim3 grid;        // stage-sweep grid of the chosen tile shape
@@ -187,7 +184,7 @@ struct F64Variant {
 constexpr F64Variant kF64Variants[] = {{32, 8}, {32, 7}, {32, 6}, {32, 4}, {16, 8}, {16, 16}, {32, 14}, {64, 7}, {8, 8}};
 // Cells above which the 8x8 tile is not tried: two per SM fill the chip there
 // and its halo (144 cells loaded for 64) can only lose (table above)
-constexpr size_t kSmallTileCells = 2 * 152 * 64;
+constexpr size_t kSmallTileCells = 2 * kSMs * 64;
 constexpr int kNumF64Variants = sizeof(kF64Variants) / sizeof(kF64Variants[0]);
 
 template <int TX, int TY, int RS = kOsher>
@@ -198,8 +195,8 @@ cudaError_t allow_f64_smem() {
 
 template <int TX, int TY, int RS = kOsher>
 cudaError_t launch_f64(const SweepArgs<double> &a, dim3 g, bool pdl, cudaStream_t s) {
-    return launch_pdl(pdl, stage_kernel<double, TX, TY, RS>, g, dim3(f64_threads(TX, TY)), sizeof(StageSmem<double, TX, TY>), s,
-                      a);
+    return launch_pdl(pdl, stage_kernel<double, TX, TY, RS>, g, dim3(f64_threads(TX, TY)),
+                      sizeof(StageSmem<double, TX, TY>), s, a);
 }
 
 // Variants that the autotuners chose, shared by the contexts of this process:
@@ -337,7 +334,7 @@ struct F64Backend : Backend {
         a.stage = stage; a.s_max = c->opt.rk_stages;
         const double dx = c->dx, dy = c->dy;
         a.dx = dx; a.dy = dy; a.half_dx = 0.5 * dx; a.half_dy = 0.5 * dy;
-        a.inv_dx = 1.0 / dx; a.inv_dy = 1.0 / dy; a.dx_over_dy = dx / dy; a.dy_over_dx = dy / dx;
+        a.dx_over_dy = dx / dy; a.dy_over_dx = dy / dx;
         a.beta = c->beta; a.inv_beta = 1.0 / c->beta; a.gx = c->grid.gx; a.gy = c->grid.gy;
         a.cfl_area = c->opt.cfl_tau * dx * dy;
         set_flux_scales(a, c->beta, dx, dy);

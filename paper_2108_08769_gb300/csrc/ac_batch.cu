@@ -71,8 +71,8 @@ __constant__ BatchTank c_tanks[kConstTanks];
 
 // Stage `stage` (coefficient alpha_s) of every active tank; blockIdx.x runs
 // over the flattened tiles.  CD: the tank's descriptor is c_tanks[slot0 + k],
-// else tanks[k].  PF: the prefetching tile sweep (see mixed_tile).  (The CTAs-per-SM hint keeps the sweep at 40 registers, see
-// ac_api.cu.)
+// else tanks[k].  PF: the prefetching tile sweep (see mixed_tile).  (The
+// CTAs-per-SM hint keeps the sweep at 40 registers, see ac_api.cu.)
 template <int TX, int TY, int NT, int RS = kOsher, bool BDF = false, bool CD = false, bool PF = false>
 __global__ void __launch_bounds__(NT, NT == 512 ? 3 : 6)
 batch_stage_kernel(const BatchTank *__restrict__ tanks, const int *__restrict__ tile_tank, int stage, float inv_alpha,
@@ -87,14 +87,16 @@ batch_stage_kernel(const BatchTank *__restrict__ tanks, const int *__restrict__ 
         if (head.done) return;
         const int local = blockIdx.x - t.tile0;
         const int by = local / t.tiles_x, bx = local - by * t.tiles_x;
-        mixed_tile<TX, TY, NT, RS, BDF, PF>(t.a, head, stage, inv_alpha, bx, by, t.a.partials + (size_t)local * 4, smem_raw);
+        mixed_tile<TX, TY, NT, RS, BDF, PF>(t.a, head, stage, inv_alpha, bx, by, t.a.partials + (size_t)local * 4,
+                                            smem_raw);
     } else {
         const BatchTank &t = tanks[k];
         const CtlHead<float> head = ctl_head<float>(t.a.ctl);
         if (head.done) return;
         const int local = blockIdx.x - t.tile0;
         const int by = local / t.tiles_x, bx = local - by * t.tiles_x;
-        mixed_tile<TX, TY, NT, RS, BDF, PF>(t.a, head, stage, inv_alpha, bx, by, t.a.partials + (size_t)local * 4, smem_raw);
+        mixed_tile<TX, TY, NT, RS, BDF, PF>(t.a, head, stage, inv_alpha, bx, by, t.a.partials + (size_t)local * 4,
+                                            smem_raw);
     }
 }
 
@@ -832,7 +834,7 @@ int ac_batch_set_state(ac_batch *b, int k, const double *rho, const double *rhou
     const ac_grid &g = b->grids[k];
     cudaStream_t s = b->stream;
     // staged in the tank's part of the two pools that do not hold its state; its buffer keeps its place
-    const int cur = b->hctl[k].cur, blocks = (int)std::min<size_t>((N + 255) / 256, 152 * 8);
+    const int cur = b->hctl[k].cur, blocks = grid_stride_blocks(N);
     const size_t o = b->off[k], fb = N * sizeof(float);
     const Staged st = staged_in(b->d[(cur + 1) % 3] + o, b->d[(cur + 2) % 3] + o, N);
     int bad = 0;
@@ -861,7 +863,7 @@ int ac_batch_get_state(const ac_batch *b, int k, double *rho, double *rhou, doub
     if (!b) return fail(AC_ERR_ARG, "batch is NULL");
     if (k < 0 || k >= b->n) return fail(AC_ERR_ARG, "tank index %d out of range", k);
     const size_t N = (size_t)b->grids[k].nx * b->grids[k].ny, o = b->off[k];
-    const int cur = b->hctl[k].cur, blocks = (int)std::min<size_t>((N + 255) / 256, 152 * 8);
+    const int cur = b->hctl[k].cur, blocks = grid_stride_blocks(N);
     double *out[4] = {rho, rhou, rhov, p};
     const Staged st = staged_in(b->d[(cur + 1) % 3] + o, b->d[(cur + 2) % 3] + o, N);
     mixed_to_fields_kernel<<<blocks, 256, 0, b->stream>>>(b->tanks_host[k].a, b->d[cur] + o, st, N);

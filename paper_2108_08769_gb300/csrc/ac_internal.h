@@ -16,9 +16,12 @@ int set_last_error(int code, const char *fmt, ...);
 // Programmatic dependent launch (AC_PDL=0 turns it off): the kernels of a
 // pseudo-iteration are launched so that each may be scheduled while its
 // predecessor in the stream is still running; every such kernel starts with
-// pdl_trigger() + pdl_wait() (ac_kernels.cuh), so it touches nothing before
-// the predecessor has finished and its writes are visible.  What overlaps is
-// the launch and CTA dispatch, not the work.
+// pdl_wait() and then pdl_trigger() (ac_kernels.cuh), so it touches nothing
+// before the predecessor has finished and its writes are visible, and lets its
+// successor in only then: a kernel waits beside its predecessor alone, which
+// is complete when the wait ends, and not beside kernels further back (the
+// other order also filled the SMs' slots unevenly, see pdl_trigger).  What
+// overlaps is the launch and CTA dispatch, not the work.
 inline bool pdl_enabled() {
     static const bool on = [] {
         const char *e = getenv("AC_PDL");
@@ -26,6 +29,10 @@ inline bool pdl_enabled() {
     }();
     return on;
 }
+
+// SMs of the GPU that grids are sized for, and the CTAs of a grid-stride pass over N cells.
+constexpr int kSMs = 152;
+inline int grid_stride_blocks(size_t N) { return (int)((N + 255) / 256 < kSMs * 8 ? (N + 255) / 256 : kSMs * 8); }
 
 // Pseudo-iterations in a captured loop's body: evaluating the loop's condition
 // costs 3 us, a tenth of a small grid's iteration (FP64 20x20, steps of 17 and

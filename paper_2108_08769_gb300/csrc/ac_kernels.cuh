@@ -87,7 +87,7 @@ struct SweepArgs {
     int gradp, limiter_k, realtime, local_dtau, alpha_pi_p_row;
     int riemann;                   // kOsher / kBassi / kRoe
     int stage, s_max;
-    T dx, dy, half_dx, half_dy, inv_dx, inv_dy, dx_over_dy, dy_over_dx;
+    T dx, dy, half_dx, half_dy, dx_over_dy, dy_over_dx;
     T beta, inv_beta, gx, gy;
     int fixed;                     // the Osher flux may run in fixed point (beta and the cell sizes allow it)
     FixedBeta fbeta;               // beta for the fixed-point Osher flux

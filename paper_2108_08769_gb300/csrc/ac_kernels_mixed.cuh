@@ -459,8 +459,8 @@ struct PrefetchSrc {
 // RAW_AUX: the ring holds (dQ of rho u, dQ of rho v, rho_ref, fold bits) as
 // copied, and the real-time terms are formed here (Backward-Euler only).
 template <int TX, int TY, int NT, int RS, bool BDF, bool RAW_AUX, typename Src>
-__device__ __forceinline__ void mixed_tile_compute(const MixedArgs &a, const CtlHead<float> &head, int stage, float inv_alpha,
-                                                   int x0, int y0, bool interior, double *partial,
+__device__ __forceinline__ void mixed_tile_compute(const MixedArgs &a, const CtlHead<float> &head, int stage,
+                                                   float inv_alpha, int x0, int y0, bool interior, double *partial,
                                                    MixedSmem<TX, TY> &sm, Src &src) {
     static_assert(!(RAW_AUX && BDF), "raw ring terms are Backward-Euler only");
     using S = MixedSmem<TX, TY>;
@@ -601,8 +601,8 @@ __device__ __forceinline__ void mixed_tile_compute(const MixedArgs &a, const Ctl
 // reference jumps are copied with cp.async while the halo is being loaded,
 // and the update's own-cell inputs are prefetched at the start of phase 3.
 template <int TX, int TY, int NT, int RS, bool BDF, bool PF = false>
-__device__ __forceinline__ void mixed_tile(const MixedArgs &a, const CtlHead<float> &head, int stage, float inv_alpha, int bx,
-                                           int by, double *partial, unsigned char *smem_raw) {
+__device__ __forceinline__ void mixed_tile(const MixedArgs &a, const CtlHead<float> &head, int stage, float inv_alpha,
+                                           int bx, int by, double *partial, unsigned char *smem_raw) {
     using S = MixedSmem<TX, TY>;
     static_assert((TX * TY) % NT == 0 && NT % 32 == 0, "tile/thread shape");
     static_assert(!PF || (NT == TX * TY && !BDF), "prefetch: one cell per thread, Backward-Euler");
@@ -845,8 +845,8 @@ struct HeldSrc {
 // windows reach ghost rows; the main loop then tests neither the row number
 // nor the fold of ghost rows.
 template <int H, int UNROLL = 1, int SK = 0>
-__device__ __forceinline__ void mixed_strip(const MixedArgs &a, const CtlHead<float> &head, int stage, float inv_alpha, int sx,
-                                            int sy, double *partial, StripRing *ring) {
+__device__ __forceinline__ void mixed_strip(const MixedArgs &a, const CtlHead<float> &head, int stage, float inv_alpha,
+                                            int sx, int sy, double *partial, StripRing *ring) {
     constexpr bool FAST = SK != 0;
     const bool st1 = SK == 0 ? (stage == 1) : (SK == 1);
     const int lane = threadIdx.x & 31;

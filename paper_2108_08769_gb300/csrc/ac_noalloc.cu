@@ -165,7 +165,7 @@ extern "C" int ac_stage_sweep_noalloc(const ac_grid *grid, double beta, const ac
     a.stage = stage; a.s_max = opt->rk_stages;
     const double dx = grid->lx / grid->nx, dy = grid->ly / grid->ny;
     a.dx = dx; a.dy = dy; a.half_dx = 0.5 * dx; a.half_dy = 0.5 * dy;
-    a.inv_dx = 1.0 / dx; a.inv_dy = 1.0 / dy; a.dx_over_dy = dx / dy; a.dy_over_dx = dy / dx;
+    a.dx_over_dy = dx / dy; a.dy_over_dx = dy / dx;
     a.beta = beta; a.inv_beta = 1.0 / beta; a.gx = grid->gx; a.gy = grid->gy;
     a.cfl_area = opt->cfl_tau * dx * dy;
     set_flux_scales(a, beta, dx, dy);
