@@ -8,11 +8,11 @@
 // evaluated in block fixed point: every quantity is a 64-bit integer and a
 // binary exponent of its own or of the face's largest term of its kind, 56 bits
 // or more of that term (FP64 keeps 53), and the sweep's other arithmetic keeps
-// the FP64 unit busy meanwhile.  A flux takes about 1770 instructions (2900
+// the FP64 unit busy meanwhile.  A flux takes about 1800 instructions (2900
 // cycles per warp with four warps on a sub-partition, near the integer
 // multiplier's rate) where the FP64 form took about 150 FP64 instructions,
 // 10,000 cycles.  One pseudo-iteration of the 256x256 tank: 193 -> 87 us, of a
-// 1024x512 tank 1440 -> 563 us (with the rest of the sweep thinned out to
+// 1024x512 tank 1440 -> 568 us (with the rest of the sweep thinned out to
 // match, see stage_kernel); the FP64 unit is then busy 42-44 % of the cycles,
 // not 80 %.  The error of 2F against 113-bit arithmetic, in units of 2^-53 of
 // its terms, is 0.3-0.9 rms where the FP64 formula's is 0.7-1.7, over the faces

@@ -308,7 +308,7 @@ struct StageSmem {
 
 // CTAs per SM the register allocation is asked to allow.  Tiles of 448 cells
 // run one per SM and take the whole register file; 256-thread tiles run three
-// (80 registers and a few spills: 558 us per pseudo-iteration of a 1024x512
+// (80 registers and a few spills: 568 us per pseudo-iteration of a 1024x512
 // tank, 660-706 us at two or four), so that the FP64-bound phases of one CTA
 // run beside the integer-bound faces of another; 128-thread tiles four.
 constexpr int f64_min_blocks(int nt) { return nt >= 448 ? 1 : nt == 256 ? 3 : nt == 128 ? 4 : 0; }
